@@ -381,12 +381,14 @@ sync_status sync_check_minimal(const sync_programs *h, sync_thr_mode mode, const
  * iteration-start costs above as described there; with licm the static time
  * bound (SYNC_PROG_OVERFLOW) adds c_wait_ops_perengine_level per cached-sum
  * update and c_regop per pair of a wait with a cached-sum read.
- * Large programs (sync_sizes.n_split_programs) whose top-level body is one
- * loop L are simulated in pieces -- runs of L's iterations -- on separate
- * warps when every wait of a piece targets an increment of the same piece
- * (checked on the thresholds of each call; otherwise, and whenever a piece
- * deadlocks or waits forward, the program is simulated whole): the barrier
- * scheme from the barrier before each piece, the barrier-free scheme by
+ * The barrier scheme is evaluated by intervals between barriers, whose
+ * schedules repeat, over all iterations at once; a program whose waits do not
+ * repeat (checked on the thresholds of each call) is walked in program order.
+ * Barrier-free, large programs (sync_sizes.n_split_programs) whose top-level
+ * body is one loop L are simulated in pieces -- runs of L's iterations -- on
+ * separate warps when every wait of a piece targets an increment of the same
+ * piece (checked on the thresholds of each call; otherwise, and whenever a
+ * piece deadlocks or waits forward, the program is simulated whole), by
  * composing the pieces' max-plus maps of the engines' cursors and last
  * retires (read off by one probe run per cursor and last retire), or, for
  * a batch of many such programs, by speculation: a piece runs from a guessed
@@ -476,9 +478,9 @@ const char *sync_last_error(void);
 /* Number of kernels this library has launched in this process, over every
  * handle, stream and thread: the loader's kernels, and per call of the
  * entry points above the kernels it enqueued (sync_simulate: one sweep and
- * one per-engine launch per call, plus the piece-parallel kernels when
- * programs are cut into pieces).  A launch counts once the CUDA runtime has
- * accepted it.  Monotonic; reading it has no other effect and cannot fail. */
+ * one per-engine launch per call, plus, when programs are cut into pieces,
+ * the piece-parallel kernels or the barrier scheme's interval kernels).  A
+ * launch counts once the CUDA runtime has accepted it.  Monotonic; reading it has no other effect and cannot fail. */
 int64_t sync_kernel_launches(void);
 
 #ifdef __cplusplus

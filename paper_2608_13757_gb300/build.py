@@ -23,9 +23,9 @@ LIB = os.path.join(LIBDIR, "libsyncgb.so")
 CUDA_HOME = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU = ["k_tiles.cu", "k_load.cu", "k_thresholds.cu", "k_simulate.cu", "k_sweep.cu", "k_piece.cu", "k_noalloc.cu"]
+CU = ["k_tiles.cu", "k_load.cu", "k_thresholds.cu", "k_simulate.cu", "k_sweep.cu", "k_bar.cu", "k_piece.cu", "k_noalloc.cu"]
 CPP = ["capi.cpp"]
-HEADERS = [os.path.join(CSRC, "enc.h"), os.path.join(CSRC, "progbuild.cuh"), os.path.join(CSRC, "cost.cuh"), os.path.join(CSRC, "sweep.cuh"), os.path.join(CSRC, "handle.h"), os.path.join(CSRC, "waitval.cuh"), os.path.join(ROOT, "include", "sync.h")]
+HEADERS = [os.path.join(CSRC, "enc.h"), os.path.join(CSRC, "progbuild.cuh"), os.path.join(CSRC, "cost.cuh"), os.path.join(CSRC, "sweep.cuh"), os.path.join(CSRC, "bar.cuh"), os.path.join(CSRC, "handle.h"), os.path.join(CSRC, "waitval.cuh"), os.path.join(ROOT, "include", "sync.h")]
 
 
 def _sources():
@@ -46,7 +46,7 @@ def _compile(src: str) -> str:
         cmd = [NVCC] + ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
                                "-Xptxas", "-warn-spills", "-c", src, "-o", obj] + inc
     else:
-        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-pthread", "-Wall", "-Wextra", "-c", src, "-o", obj,
+        cmd = ["g++", "-O3", "-std=c++17", "-fPIC", "-pthread", "-Wall", "-Wextra", "-c", src, "-o", obj,
                "-I", os.path.join(CUDA_HOME, "include")] + inc
     subprocess.check_call(cmd)
     return obj

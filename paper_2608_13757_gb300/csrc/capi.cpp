@@ -4,13 +4,16 @@
 #include <algorithm>
 #include <array>
 #include <atomic>
+#include <condition_variable>
 #include <cstdlib>
 #include <cstring>
 #include <exception>
+#include <functional>
 #include <memory>
 #include <mutex>
 #include <new>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <unordered_map>
 #include <utility>
@@ -210,6 +213,7 @@ void check_totals(const int64_t* count) {
   if (count[BC_OPS] > kI32Max) raise(SYNC_ERR_OVERFLOW, "op records exceed INT32_MAX entries");
   if (count[BC_PLAN] > kI32Max || count[BC_CHUNKS] > kI32Max || count[BC_LANES] > kI32Max)
     raise(SYNC_ERR_OVERFLOW, "sweep tables exceed INT32_MAX entries");
+  if (count[BC_TILES] > kI32Max - 1) raise(SYNC_ERR_OVERFLOW, "interval tiles exceed INT32_MAX entries");
 }
 
 }  // namespace
@@ -230,8 +234,7 @@ static int64_t split_floor() {
 // environment variable SYNCGB_SPLIT_MIN sets another floor) and
 // more than 8 times the instances per resident sweep warp (152 SMs x 24
 // warps on a GB300) of the whole batch, so that its serial walk, not the
-// batch's throughput, bounds the simulation (the barrier scheme runs each
-// piece twice).  Barrier-free, a program is probed (2*ne runs per piece)
+// batch's throughput, bounds the barrier-free simulation.  A program is probed (2*ne runs per piece)
 // when it stays above 4 * (2*ne + 1) times that share, and speculated
 // otherwise (SYNCGB_SPLIT_SPEC=1 speculates always).
 static void build_pieces(const sync_batch_desc& d, const LoopInfo* loop, const int32_t* rowptr, const int4* xsem,
@@ -249,7 +252,7 @@ static void build_pieces(const sync_batch_desc& d, const LoopInfo* loop, const i
   std::vector<VDep> vdep;
   std::vector<int32_t> pub, cnt, bf_init;
   int64_t hist_split[kModes] = {0, 0, 0};
-  int64_t inst_bb = 0, inst_bf = 0;               // compact instance spaces (barrier scheme, barrier-free)
+  int64_t inst_bb = 0, inst_bf = 0;               // compact instance spaces (all, probed)
   int32_t ne_max = 0;
   std::vector<int32_t> path, row;
   for (int32_t p = 0; p < P; ++p) {
@@ -394,8 +397,8 @@ namespace {
 // Each load takes one of each from a pool and gives it back; a pinned arena
 // is reused only after the copy out of it has completed (its event).
 struct HostScratch {
-  HostVec<int32_t> i32_nl[2], body_ptr, body, i32_nx[6], i32_rows[2], anc, i32_nd[3];
-  HostVec<uint8_t> u8_nl[2], rpflag, dep_bar;
+  HostVec<int32_t> i32_nl[3], body_ptr, body, i32_nx[8], i32_rows[4], anc, i32_nd[5];
+  HostVec<uint8_t> u8_nl[3], rpflag, dep_bar, dep_fix;
   HostVec<int64_t> keys, i64_rows[3], ord_off, count, base;
   HostVec<uint32_t> pe_of;
   HostVec<Seen> seen;
@@ -472,32 +475,91 @@ T* sized(HostVec<T>& v, int64_t n) {
   return v.data();
 }
 
-// Runs f(p) for programs [0, P) on host threads, in contiguous blocks.
-template <class F>
-void for_programs(int32_t P, F f) {
-  const int n_threads = load_threads(P);
-  std::vector<std::thread> pool;
-  std::vector<std::exception_ptr> err(n_threads);
-  for (int t = 0; t < n_threads; ++t) {
-    const int32_t b = (int32_t)((int64_t)P * t / n_threads), e = (int32_t)((int64_t)P * (t + 1) / n_threads);
-    auto job = [&f, &err, t, b, e] {
+// The host threads of one load: started once and used by both passes (a
+// chain load of 8192 programs spent 0.3 ms a pass on starting and joining 16
+// threads).  A thread that cannot be started is done without.
+class Team {
+ public:
+  explicit Team(int n) {
+    for (int t = 1; t < n; ++t) {
       try {
-        for (int32_t p = b; p < e; ++p) f(p);
-      } catch (...) {
-        err[t] = std::current_exception();
+        pool_.emplace_back([this, t] { work(t); });
+      } catch (const std::system_error&) {
+        break;
       }
-    };
-    if (t + 1 < n_threads) pool.emplace_back(job); else job();
+    }
+    err_.resize(pool_.size() + 1);
   }
-  for (auto& th : pool) th.join();
-  for (auto& x : err)
-    if (x) std::rethrow_exception(x);
-}
+  ~Team() {
+    {
+      std::lock_guard<std::mutex> g(mu_);
+      stop_ = true;
+    }
+    go_.notify_all();
+    for (auto& th : pool_) th.join();
+  }
+  Team(const Team&) = delete;
+  Team& operator=(const Team&) = delete;
+
+  // f(p) for programs [0, P), in contiguous blocks
+  template <class F>
+  void for_programs(int32_t P, F f) {
+    const int n = (int)pool_.size() + 1;
+    const std::function<void(int)> job = [&](int t) {
+      const int32_t b = (int32_t)((int64_t)P * t / n), e = (int32_t)((int64_t)P * (t + 1) / n);
+      for (int32_t p = b; p < e; ++p) f(p);
+    };
+    {
+      std::lock_guard<std::mutex> g(mu_);
+      job_ = &job;
+      running_ = n - 1;
+      ++turn_;
+    }
+    go_.notify_all();
+    run(0);
+    std::unique_lock<std::mutex> g(mu_);
+    done_.wait(g, [this] { return running_ == 0; });
+    for (auto& x : err_)
+      if (x) std::rethrow_exception(std::exchange(x, nullptr));
+  }
+
+ private:
+  void run(int t) {
+    try {
+      (*job_)(t);
+    } catch (...) {
+      err_[t] = std::current_exception();
+    }
+  }
+  void work(int t) {
+    uint64_t seen = 0;
+    for (;;) {
+      {
+        std::unique_lock<std::mutex> g(mu_);
+        go_.wait(g, [&] { return stop_ || turn_ != seen; });
+        if (stop_) return;
+        seen = turn_;
+      }
+      run(t);
+      std::lock_guard<std::mutex> g(mu_);
+      if (--running_ == 0) done_.notify_one();
+    }
+  }
+
+  std::vector<std::thread> pool_;
+  std::vector<std::exception_ptr> err_;
+  std::mutex mu_;
+  std::condition_variable go_, done_;
+  const std::function<void(int)>* job_ = nullptr;
+  uint64_t turn_ = 0;
+  int running_ = 0;
+  bool stop_ = false;
+};
 
 // COUNT over the covered programs on host threads (validation, counts and
 // summaries), the first failure reported as the loader reports it, then the
 // exclusive prefix sums of the counts; returns the totals.
-void count_pass(const sync_batch_desc& d, const Shape& sh, HostScratch& H, BuildArgs& a,
+void count_pass(const sync_batch_desc& d, const Shape& sh, Team& team, HostScratch& H, BuildArgs& a,
                 int64_t tot[kBuildCounts]) {
   const int32_t P = sh.P, Pq = sh.covered;
   const int64_t NL = sh.NL, NX = sh.NX, ND = sh.ND, rows = sh.rows;
@@ -516,15 +578,20 @@ void count_pass(const sync_batch_desc& d, const Shape& sh, HostScratch& H, Build
   BuildScratch& S = a.s;
   S.depth = sized(H.i32_nl[0], NL);
   S.lfill = sized(H.i32_nl[1], NL);
+  S.cidx = sized(H.i32_nl[2], NL);
   S.needs_rhat = sized(H.u8_nl[0], NL);
   S.fbar = sized(H.u8_nl[1], NL);
+  S.unit = sized(H.u8_nl[2], NL);
   S.body_ptr = sized(H.body_ptr, NL + P);
   S.keys = sized(H.keys, NX + NL);
   S.body = sized(H.body, NX + NL);
-  int32_t** nx_arrays[6] = {&S.rank, &S.x_ndeps, &S.x_dep_begin, &S.x_levels, &S.cons_next, &S.sem_x};
-  for (int i = 0; i < 6; ++i) *nx_arrays[i] = sized(H.i32_nx[i], NX);
+  int32_t** nx_arrays[8] = {&S.rank,      &S.x_ndeps, &S.x_dep_begin, &S.x_levels,
+                            &S.cons_next, &S.sem_x,   &S.op_of,       &S.prevc};
+  for (int i = 0; i < 8; ++i) *nx_arrays[i] = sized(H.i32_nx[i], NX);
   S.nloop_eng = sized(H.i32_rows[0], rows);
   S.sem_row = sized(H.i32_rows[1], rows);
+  S.fix_cnt = sized(H.i32_rows[2], rows);
+  S.before = sized(H.i32_rows[3], rows);
   int64_t** row_arrays[3] = {&S.stot, &S.srp, &S.tstart};
   for (int i = 0; i < 3; ++i) *row_arrays[i] = sized(H.i64_rows[i], rows);
   S.pe_of = sized(H.pe_of, rows);
@@ -534,11 +601,14 @@ void count_pass(const sync_batch_desc& d, const Shape& sh, HostScratch& H, Build
   S.dep_S = sized(H.i32_nd[0], ND);
   S.dep_N = sized(H.i32_nd[1], ND);
   S.by_cons = sized(H.i32_nd[2], ND);
+  S.dep_ca = sized(H.i32_nd[3], ND);
+  S.dep_cb = sized(H.i32_nd[4], ND);
+  S.dep_fix = sized(H.dep_fix, ND);
   S.seen = sized(H.seen, ND);
   a.o.ord_off = sized(H.ord_off, NX);          // COUNT's dedup marks
   a.count = sized(H.count, (int64_t)Pq * kBuildCounts);
   a.sum = sized(H.sum, Pq);
-  for_programs(Pq, [&a](int32_t p) {
+  team.for_programs(Pq, [&a](int32_t p) {
     ProgBuilder<false> b(a, p);
     b.run();
   });
@@ -608,7 +678,8 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   ScratchLease SL;
   BuildArgs a{};
   int64_t cnt[kBuildCounts];
-  count_pass(d, sh, *SL.s, a, cnt);
+  Team team(load_threads(P));
+  count_pass(d, sh, team, *SL.s, a, cnt);
   cuda_check(cudaSetDevice(device), "cudaSetDevice");
   h.device = device;
   cuda_check(cudaDeviceGetAttribute(&h.num_sms, cudaDevAttrMultiProcessorCount, device), "device attributes");
@@ -617,7 +688,6 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   const int64_t n_ops = cnt[BC_OPS], n_plan = cnt[BC_PLAN], n_lanes = cnt[BC_LANES];
   const int64_t n_iters = cnt[BC_ITERS], n_derived = cnt[BC_DERIVED], n_jobs = cnt[BC_JOBS];
   const int64_t n_pairs_padded = cnt[BC_PADDED];
-  const int64_t n_xloops = div ? rows : NL;
   int64_t hist_max = 0;
   for (int m = 0; m < kModes; ++m) hist_max = std::max(hist_max, h.hist_len[m] = cnt[BC_HIST + m]);
   const int64_t n_first_tiles = (n_pairs_padded + kTilePairs - 1) / kTilePairs;
@@ -631,17 +701,21 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   const size_t o_dsem = L.add<int32_t>(kModes * ND), o_lflag = L.add<int32_t>(NL);
   const size_t o_plan_ptr = L.add<int32_t>(NL + 1), o_op_ptr = L.add<int32_t>(rows + 1);
   const size_t o_rowinfo = L.add<int2>(rows), o_hoist = L.add<int32_t>(rows);
-  const size_t o_xloops = L.add<LoopInfo>(n_xloops), o_reads = L.add<uint8_t>(n_xloops);
   const size_t o_rowptr = L.add<int32_t>(cnt[BC_ROWPTR]), o_path = L.add<int64_t>(cnt[BC_PATH]);
   const size_t o_jobs = L.add<DeriveJob>(n_jobs), o_ops = L.add<int4>(n_ops), o_opstop = L.add<int32_t>(n_ops);
   const size_t o_semhb = L.add<int64_t>(cnt[BC_SEMHB]), o_plan = L.add<int4>(n_plan), o_paux = L.add<int4>(n_plan);
   const size_t o_chunks = L.add<int4>(cnt[BC_CHUNKS]), o_lrec = L.add<int4>(n_lanes), o_lmeta = L.add<int4>(n_lanes);
-  const size_t o_order = L.add<int32_t>(P);
+  const size_t o_order = L.add<int32_t>(P), o_bl = L.add<BarLoop>(NL + 1), o_bdep = L.add<BarDep>(ND);
+  const size_t o_rowc = L.add<int2>(rows);
   const size_t host_bytes = L.bytes;
   const size_t o_derived = L.add<int32_t>(n_derived);
   const size_t o_opsem = L.add<int4>(kModes * n_ops), o_lsem = L.add<int4>(kModes * n_lanes);
-  const size_t o_hist = L.add<int32_t>(hist_max), o_slot = L.add<int32_t>(1), o_fallback = L.add<int32_t>((int64_t)P + 1);
+  const size_t o_hist = L.add<int32_t>(hist_max), o_slot = L.add<int32_t>(kCounters + (int64_t)P);
   const size_t o_tile_first = L.add<int32_t>(n_first_tiles + 1), o_tile_job = L.add<int32_t>(n_job_tiles + 1);
+  const int64_t n_tiles = cnt[BC_TILES];
+  const size_t o_tile_loop = L.add<int32_t>(n_tiles + 1), o_F = L.add<int32_t>(cnt[BC_FPOOL]);
+  const size_t o_rel = L.add<int2>(n_ops), o_ko = L.add<int2>(NL), o_bind = L.add<uint8_t>(ND);
+  const size_t o_left = L.add<int32_t>(P), o_counted = L.add<int32_t>(P), o_todo = L.add<int32_t>((int64_t)P + 1);
   char* dev = h.alloc<char>((int64_t)L.bytes, "encoding");
 
   // ------------------------------------------------------------- FILL
@@ -666,8 +740,6 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   O.op_ptr = reinterpret_cast<int32_t*>(host + o_op_ptr);
   O.rowinfo = reinterpret_cast<int2*>(host + o_rowinfo);
   O.hoist = reinterpret_cast<int32_t*>(host + o_hoist);
-  O.xloops = reinterpret_cast<LoopInfo*>(host + o_xloops);
-  O.reads_rowptr = reinterpret_cast<uint8_t*>(host + o_reads);
   O.rowptr = reinterpret_cast<int32_t*>(host + o_rowptr);
   O.path = reinterpret_cast<int64_t*>(host + o_path);
   O.jobs = reinterpret_cast<DeriveJob*>(host + o_jobs);
@@ -679,12 +751,16 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   O.chunks = reinterpret_cast<int4*>(host + o_chunks);
   O.lrec = reinterpret_cast<int4*>(host + o_lrec);
   O.lmeta = reinterpret_cast<int4*>(host + o_lmeta);
+  O.bl = reinterpret_cast<BarLoop*>(host + o_bl);
+  O.bdep = reinterpret_cast<BarDep*>(host + o_bdep);
+  O.rowc = reinterpret_cast<int2*>(host + o_rowc);
+  O.bl[NL] = BarLoop{};
   // the closing entries of the offset tables: 0 without programs, else the
   // last program's FILL writes them
   O.seg[ND] = 0;
   O.op_ptr[rows] = 0;
   O.plan_ptr[NL] = 0;
-  for_programs(P, [&a](int32_t p) {
+  team.for_programs(P, [&a](int32_t p) {
     ProgBuilder<true> b(a, p);
     b.run();
   });
@@ -728,7 +804,28 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   h.lsem = reinterpret_cast<int4*>(D(o_lsem));
   h.hist = reinterpret_cast<int32_t*>(D(o_hist));
   h.next_slot = reinterpret_cast<int32_t*>(D(o_slot));
-  h.fallback = reinterpret_cast<int32_t*>(D(o_fallback));
+  h.fallback = h.next_slot + kCounters - 1;
+  BarArgs& b = h.bar;
+  b.on = div ? 0 : 1;
+  b.n_tiles = (int32_t)n_tiles;
+  b.bl = reinterpret_cast<BarLoop*>(D(o_bl));
+  b.bdep = reinterpret_cast<BarDep*>(D(o_bdep));
+  b.rowc = reinterpret_cast<int2*>(D(o_rowc));
+  b.tile_loop = reinterpret_cast<int32_t*>(D(o_tile_loop));
+  b.op_ptr = h.op_ptr;
+  b.ops = h.ops;
+  b.dep = h.dep;
+  b.ddep = h.ddep;
+  b.path = h.path;
+  b.derived = h.derived;
+  b.rel = reinterpret_cast<int2*>(D(o_rel));
+  b.ko = reinterpret_cast<int2*>(D(o_ko));
+  b.bind = reinterpret_cast<uint8_t*>(D(o_bind));
+  b.F = reinterpret_cast<int32_t*>(D(o_F));
+  b.left = reinterpret_cast<int32_t*>(D(o_left));
+  b.counted = reinterpret_cast<int32_t*>(D(o_counted));
+  b.plans = h.next_slot + 1;
+  h.todo = reinterpret_cast<int32_t*>(D(o_todo));
   h.tile_first = reinterpret_cast<int32_t*>(D(o_tile_first));
   const DeriveJob* d_jobs = reinterpret_cast<const DeriveJob*>(D(o_jobs));
   int32_t* tile_job = reinterpret_cast<int32_t*>(D(o_tile_job));
@@ -742,6 +839,7 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
     code_looped += s.code_looped;
     code_unrolled += s.code_unrolled;
     n_bar_deps += s.n_bar_deps;
+    h.max_inst = std::max(h.max_inst, s.n_inst);
     ne_max = std::max(ne_max, s.ne);
     depth_max = std::max(depth_max, s.depth_max);
     ord_overflow |= s.ord_overflow;
@@ -787,13 +885,14 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
 
   // ----------------------------------------------------------- device
   cuda_check(launch_tile_tables(h.seg, ND, h.tile_first, n_first_tiles, d_jobs, n_jobs, tile_job, n_job_tiles,
-                                h.num_sms, stream),
+                                h.bar.bl, NL, const_cast<int32_t*>(h.bar.tile_loop), n_tiles, h.num_sms, stream),
              "tile tables");
   cuda_check(launch_sem_records(reinterpret_cast<const int4*>(D(o_xsem)), NX, h.ops, n_ops, h.lrec, n_lanes, h.opsem,
                                 h.lsem, h.num_sms, stream),
              "semaphore records");
   cuda_check(launch_derive(d_jobs, tile_job, n_drows, h.rowptr, h.path, h.derived, n_derived, h.num_sms, stream),
              "derive");
+  cuda_check(cudaMemsetAsync(h.bar.counted, 0, sizeof(int32_t) * (size_t)P, stream), "interval counts");
   cuda_check(cudaEventCreateWithFlags(&h.ready, cudaEventDisableTiming), "load event");
   cuda_check(cudaEventRecord(h.ready, stream), "load event");
 }
@@ -804,7 +903,8 @@ static void validate(const sync_batch_desc& d) {
   ScratchLease SL;
   BuildArgs a{};
   int64_t tot[kBuildCounts];
-  count_pass(d, sh, *SL.s, a, tot);
+  Team team(load_threads(sh.covered));
+  count_pass(d, sh, team, *SL.s, a, tot);
 }
 
 
@@ -959,13 +1059,13 @@ static int32_t* probe_history(const sync_programs* h, sync_thr_mode mode) {
 }
 
 // The stored times of the piece runs: per instance of the split programs
-// (barrier-free: of the ones split barrier-free) issue and retire per run
+// (single runs: all of them, else the probed ones) issue and retire per run
 // and the position in its engine's stream; allocated on first use.
-static int32_t* stored_times(const sync_programs* h, bool barrier) {
+static int32_t* stored_times(const sync_programs* h, bool single) {
   std::lock_guard<std::mutex> lock(h->phist_mu);
-  const int k = barrier ? 0 : 1;
+  const int k = single ? 0 : 1;
   if (!h->ptimes[k]) {
-    const int64_t runs = barrier ? 1 : h->probes_bf;
+    const int64_t runs = single ? 1 : h->probes_bf;
     h->ptimes[k] = h->alloc_lazy<int32_t>((2 * runs + 1) * std::max<int64_t>(h->pinst[k], 1), "piece times");
   }
   return h->ptimes[k];
@@ -1042,9 +1142,21 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
   w.dep = a.dep; w.ddep = a.ddep; w.path = a.path; w.ord = a.ord;
   w.chk_counts = a.chk_counts; w.chk_first = a.chk_first;
   const bool barrier = variant == SYNC_SIM_BARRIER;
-  // split programs (array thresholds): simulated piece by piece on many warps
-  // first; the sweep skips the ones the pieces completed
-  if (!fused && h->n_split > 0) {
+  // barrier scheme (array thresholds): by intervals, in the sweep's launch or,
+  // with split programs, in launches of its own
+  if (!fused && barrier && h->bar.on && h->max_inst >= kBarMinInst) {
+    w.bar = h->bar;
+    if (const int r = sweep_ring_for(a.sem_cap, a.frame_depth, kBarRingBytes)) w.ring = r;
+    w.bar.min_inst = kBarMinInst;
+    if (h->n_split > 0) {
+      cuda_check(launch_intervals(w, h->todo, h->sz.n_loops, st), "interval simulation");
+      w.bar.on = 0;
+      w.bar.todo = h->todo;
+    }
+  }
+  // split programs barrier-free (array thresholds): simulated piece by piece
+  // on many warps first; the sweep skips the ones the pieces completed
+  if (!fused && !barrier && h->n_split > 0) {
     cuda_check(cudaMemsetAsync(h->piece_fail, 0, sizeof(int32_t) * (size_t)h->n_split, st), "cudaMemsetAsync");
     w.pcs.piece = h->pieces; w.pcs.split = h->splits; w.pcs.prog_split = h->prog_split;
     w.pcs.pub = h->piece_pub; w.pcs.fail = h->piece_fail; w.pcs.out = h->piece_out; w.pcs.x = h->piece_x;
@@ -1055,21 +1167,15 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
     w.pcs.cls = h->piece_cls; w.pcs.need = h->spec_need; w.pcs.has = h->spec_has; w.pcs.xhat = h->spec_xhat;
     w.pcs.shift = h->piece_shift; w.pcs.vp = h->spec_vp;
     SweepArgs wp = w;
-    PieceLaunch L{h->vdep, h->piece_cnt, stored_times(h, true), h->pinst[0], h->n_split, 0, 0};
-    if (barrier) {
-      wp.pcs.probes = 1;
-    } else {
-      L.n_probed = h->n_probed;
-      L.n_spec = h->n_spec;
-      wp.pcs.probes = h->probes_bf;
-      if (h->n_probed > 0) {                       // the probes' histories and stored times
-        wp.pcs.phist = probe_history(h, mode);
-        wp.pcs.phist_len = h->phist_len[mode];
-        wp.pcs.ptimes = stored_times(h, false);
-        wp.pcs.plen = h->pinst[1];
-      }
+    PieceLaunch L{h->vdep, h->piece_cnt, stored_times(h, true), h->pinst[0], h->n_split, h->n_probed, h->n_spec};
+    wp.pcs.probes = h->probes_bf;
+    if (h->n_probed > 0) {                         // the probes' histories and stored times
+      wp.pcs.phist = probe_history(h, mode);
+      wp.pcs.phist_len = h->phist_len[mode];
+      wp.pcs.ptimes = stored_times(h, false);
+      wp.pcs.plen = h->pinst[1];
     }
-    cuda_check(launch_pieces(wp, barrier, L, h->num_sms, st), "piece simulation");
+    cuda_check(launch_pieces(wp, L, h->num_sms, st), "piece simulation");
   }
   cuda_check(launch_sweep(w, barrier, h->num_sms, st), "sweep simulator kernel");
   a.only = h->fallback;

@@ -82,6 +82,9 @@ struct alignas(16) ProgInfo {
   int32_t semhb_off[kModes];  // first entry of the program's history bases, per mode
   int32_t loop_base;  // global id of the program's top-level loop
   int32_t divergent;  // 1: engines run their own trip counts (per-engine kernel only)
+  int32_t nloops;
+  int32_t dep0, ndep; // its consumer-grouped dependencies [dep0, dep0 + ndep)
+  int32_t pad_;
 };
 
 // Program-order sweep tables.  Per loop, a plan: its body cut at child loops
@@ -209,9 +212,7 @@ struct CostTables {
 // instance counts and each waited semaphore's published increments at its
 // start.  Per call: a validation that every wait of a piece targets an
 // increment the piece itself produces (else the program is simulated whole),
-// then barrier scheme: one run per piece from a barrier release at 0 and a
-// prefix sum of the piece durations; barrier-free: the piece's end state
-// (engine cursors and last retires) is a max-plus linear map of its start
+// then the piece's end state (engine cursors and last retires) is a max-plus linear map of its start
 // state, read off by one probe run per state variable (the variable raised
 // by kProbe, the others 0), composed piece by piece.  The runs store every
 // instance's times, from which a last pass forms the true ones.
@@ -219,8 +220,8 @@ constexpr int32_t kProbe = 1 << 30;         // probe offset; split programs' tim
 
 struct alignas(16) PieceInfo {
   int64_t hdelta[kModes];   // probe runs: history entry = semhb + hdelta + probe * probe_hist_len[mode]
-  int64_t tl[2];            // compact scratch index of instance o = o + tl[0] (barrier scheme: every
-                            // split program) or o + tl[1] (barrier-free: the ones split barrier-free)
+  int64_t tl[2];            // compact scratch index of instance o = o + tl[0] (single runs: every split
+                            // program) or o + tl[1] (probes: the probed ones)
   int32_t prog, split;      // program id, its index among the split programs
   int32_t loop, g0, g1;     // iterations [g0, g1) of L (global loop id and iteration indices)
   int32_t pub_off[kModes];  // published increments at the start, per waited semaphore (pool pub)
@@ -277,6 +278,89 @@ struct PieceArgs {
   int32_t* shift;           // [n_pieces]: accepted pieces: true times - stored times
   int32_t* vp;              // [n_split]: pieces accepted so far
 };
+
+// Interval tables (bar.cuh): the barrier scheme cuts a program's run at its
+// barriers into intervals that start with every engine at one time and
+// everything earlier retired, so an interval's schedule is fixed by its
+// segment alone, and start times and engine-stream positions are sums of
+// per-loop constants over the trip prefix sums.  A loop that runs exactly
+// once on every visit, and whose child loops do (`fixed`), is part of its
+// parent's iteration: its host is the nearest loop around it that is not.
+struct alignas(16) BarLoop {   // per loop, and a last entry (tile0: all tiles)
+  int64_t foff;      // a loop with child loops that are not fixed: its arrays in the pool F, -1 otherwise.
+                     // Per quantity q (0 time, 1 + e instances of engine e) [total] starts of its
+                     // iterations, then per quantity [total + 1] sums over its first iterations
+  int32_t prog;
+  int32_t item;      // its plan item in its parent's body
+  int32_t host;      // itself unless fixed
+  int32_t nchild;    // child loops that are not fixed
+  int32_t esib;      // such loops before it in its parent's body
+  int32_t tile0;     // its first tile
+  int32_t iters;     // iterations per tile (a multiple of 32)
+  int32_t pad_;
+};
+// Per consumer-grouped dependency (producer p in loop P, consumer in loop C,
+// innermost common loop S, boundary = start of the consumer's straight-line
+// segment, or of S's child towards C): the increments published at the
+// boundary are, with gs the consumer's S-iteration, X = gs (P = S) or the
+// iterations of P through S-iteration gs - 1 + delta:
+//   count X + b[0]; per loop N*X + b[1]; per engine the engine's instances
+//   before C's iteration and its children so far + b2.
+struct alignas(16) BarDep {
+  int32_t prod_op;   // op record of a producer in the consumer's own segment, else -1
+  int32_t b[2];
+  int32_t b2;
+  int32_t cons_loop; // C
+  int32_t cons_item; // plan item of the last child loop of C before the consumer, or -1
+  uint8_t ep;        // producer's engine
+  uint8_t delta;
+  uint8_t cons_fixed;  // S's iteration is C's (only fixed loops between)
+  uint8_t prod_fixed;  // X = gs + delta (likewise)
+  int32_t pad_;
+};
+struct BarArgs {
+  int32_t on;                // 1: the sweep launch runs the intervals first (bar.cuh)
+  int32_t n_tiles;
+  int32_t min_inst;          // programs with fewer instances are swept
+  const BarLoop* bl;
+  const BarDep* bdep;
+  const int2* rowc;          // per (loop, engine): instances {before it in its parent's (fixed: its host's)
+                             // iteration, in one iteration}, loops that are not fixed excluded
+  const int32_t* tile_loop;  // [n_tiles]
+  const int32_t* op_ptr;
+  const int4* ops;
+  const DepInfo* dep;
+  const int32_t* ddep;
+  const int64_t* path;
+  const int32_t* derived;
+  int2* rel;                 // scratch per op record: issue, retire from its iteration's start
+  int2* ko;                  // scratch per loop: {duration of an iteration, offset in its parent's},
+                             // both without the child loops' own durations
+  uint8_t* bind;             // scratch per grouped dependency: 1 = waits inside its interval
+  int32_t* F;
+  int32_t* left;             // scratch per program: tiles left; kBarBad: a wait differs; < 0: not by intervals
+  int32_t* counted;          // per program, zeroed at load: 1 = its counts (q >= 1) are in F
+  int32_t* plans;            // zeroed per call: programs planned
+  const int32_t* todo;       // sweep only these: [0] count, [1..] programs (NULL: all)
+};
+constexpr int32_t kBarBad = 1 << 30;
+// Programs with fewer instances are swept: a plan is a chain of about 30 us,
+// what the walk takes for 300 instances (one program of 96: 18 us swept, 36
+// by intervals).
+constexpr int32_t kBarMinInst = 256;
+constexpr size_t kBarRingBytes = 32 * 1024;
+// Counters a sweep launch starts from, zeroed together: next_slot[0], the
+// intervals' count of planned programs, fallback[0] (the list follows).
+constexpr int32_t kCounters = 3;
+// Iterations of a tile: 2048 to 4096 instances in steps of 128 iterations
+// (what a warp takes at a time, 4 per lane); 32 for a loop with moving
+// children, whose iterations are few and long, and for a long body, one of
+// which fills a warp's time.
+constexpr inline int32_t bar_iters(int64_t records, int64_t moving) {
+  if (moving > 0 || records > 64) return 32;
+  const int64_t w = records > 0 ? 16 / records : 4;
+  return 128 * (int32_t)(w < 1 ? 1 : w > 4 ? 4 : w);
+}
 
 struct SimArgs {
   const ProgInfo* prog;
@@ -361,6 +445,7 @@ struct SweepArgs {
   unsigned long long* chk_first;   // optional: [1] smallest offending pair index
   CostTables cost;
   PieceArgs pcs;             // piece-parallel simulation (prog_split NULL: none)
+  BarArgs bar;               // barrier scheme by intervals
 };
 
 // Launchers (return the launch error, if any).
@@ -391,19 +476,22 @@ cudaError_t launch_simulate(const SimArgs& a, bool barrier, int num_sms, cudaStr
 // the per-engine kernel (launch_simulate with SimArgs::only set).
 cudaError_t launch_sweep(const SweepArgs& a, bool barrier, int num_sms, cudaStream_t s);
 size_t sweep_smem_bytes(int sem_cap, int frame_depth, int ring);
-// Piece-parallel simulation of the split programs (a.pcs): validation, the
-// probe (barrier-free) or relative (barrier) runs, the composition of the
-// pieces, and the pass that forms the instances' true times (checksums,
+// Piece-parallel simulation of the split programs (a.pcs), barrier-free:
+// validation, the probe runs or speculation, the composition of the pieces, and the pass that forms the instances' true times (checksums,
 // timelines); the programs it completes are marked in a.pcs.fail (0) for
 // launch_sweep to skip.
 struct PieceLaunch {
   const VDep* vdep;
   const int32_t* cnt;
-  int32_t* one;              // stored times of single runs (barrier scheme, speculation)
+  int32_t* one;              // stored times of single runs (speculation)
   int64_t one_len;           // instances of all split programs
   int32_t n_split, n_probed, n_spec;   // split programs; of these barrier-free probed / speculated
 };
-cudaError_t launch_pieces(const SweepArgs& a, bool barrier, const PieceLaunch& L, int num_sms, cudaStream_t s);
+cudaError_t launch_pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaStream_t s);
+// Barrier scheme by intervals in separate launches, for a batch with split
+// programs (their loops are scheduled by separate warps); programs it
+// cannot do are listed in todo for launch_sweep.
+cudaError_t launch_intervals(const SweepArgs& a, int32_t* todo, int32_t n_loops, cudaStream_t s);
 // Largest ring (32, 16, ..., 1) whose sweep shared memory fits in `limit`
 // bytes, or 0 if none does.
 int sweep_ring_for(int sem_cap, int frame_depth, size_t limit);

@@ -85,6 +85,9 @@ struct sync_programs {
   int32_t* hist = nullptr;          // scratch: retire time of each semaphore increment
   int32_t* next_slot = nullptr;     // scratch: simulator's program-slot counter
   int32_t* fallback = nullptr;      // scratch: programs handed to the per-engine kernel
+  int64_t max_inst = 0;             // instances of the largest program
+  syncgb::BarArgs bar{};            // barrier scheme by intervals (bar.cuh)
+  int32_t* todo = nullptr;          // scratch: programs the intervals leave to the sweep
   // program-order sweep
   int32_t* plan_ptr = nullptr;
   int4* plan = nullptr;
@@ -115,7 +118,7 @@ struct sync_programs {
   int64_t phist_len[syncgb::kModes] = {0, 0, 0};   // probe history entries per probe, per mode
   mutable std::mutex phist_mu;
   mutable int32_t* phist[syncgb::kModes] = {nullptr, nullptr, nullptr};   // allocated on first use
-  int64_t pinst[2] = {0, 0};            // instances of the split programs (barrier scheme, barrier-free)
+  int64_t pinst[2] = {0, 0};            // instances of the split programs (all, probed)
   mutable int32_t* ptimes[2] = {nullptr, nullptr};   // their stored times, allocated on first use
   int32_t* xeng = nullptr;              // engine per instruction (split batches)
   int32_t nx_max_split = 1;             // most instructions of a split program

@@ -12,20 +12,18 @@
 //   - under the timing model every time in a piece is the maximum, over
 //     paths from those start values, of a start value plus a sum of costs
 //     (all costs >= 0, no constant terms), so the piece's end state is a
-//     max-plus linear map of its start state.  Barrier scheme: a barrier
-//     release precedes every piece (every engine at the release time, the
-//     last retires below it), so the map is a shift by the piece's duration.
-//     Barrier-free: probe q runs the piece with state variable q at kProbe
-//     and the others at 0; since no path weight reaches kProbe (the time
-//     bound of a split program is below it), output o of probe q is
-//     kProbe + M[o][q] when o depends on q and below kProbe otherwise.
+//     max-plus linear map of its start state.  Probe q runs the piece with
+//     state variable q at kProbe and the others at 0; since no path weight
+//     reaches kProbe (the time bound of a split program is below it), output
+//     o of probe q is kProbe + M[o][q] when o depends on q and below kProbe
+//     otherwise.
 // The pieces of a program are then composed in order (x_{j+1} = M_j x_j).  The
 // same linearity holds for every instance's issue and retire times, which
 // the piece runs store (per probe, with the instance's position in its
 // engine's stream): a memory-bound pass then forms the true times from the
-// start states -- shifted by the piece's start (barrier scheme), or the
-// maximum over the probes of stored time - kProbe + start value (barrier-
-// free) -- for the checksum and the timelines.
+// start states, the maximum over the probes of stored time - kProbe + start
+// value, for the checksum and the timelines.  The barrier scheme needs no
+// pieces (bar.cuh).
 #include <algorithm>
 
 #include "sweep.cuh"
@@ -41,7 +39,7 @@ constexpr int kSpecRounds = 4;              // rounds of speculation before a pr
 // semaphore's published increments at the piece start.  The first piece of
 // a program also checks the program's static time bound (below kProbe for
 // the probes; the sweep reports an overflow itself).
-template <int MODE, bool BB>
+template <int MODE>
 __global__ void __launch_bounds__(kValThreads) k_piece_validate(const SweepArgs a, const VDep* __restrict__ vdep,
                                                                 const int32_t* __restrict__ cnt) {
   const int piece = blockIdx.x;
@@ -51,7 +49,7 @@ __global__ void __launch_bounds__(kValThreads) k_piece_validate(const SweepArgs 
   const int j = piece - sp.first_piece;
   if (j == 0 && threadIdx.x == 0) {
     const int32_t cwait = MODE == SYNC_THR_COUNT ? a.prm.c_wait_ops_count : a.prm.c_wait_ops_perloop;
-    if (time_bound<MODE, BB>(a.prog[pc.prog], a.prm, cwait) >= (unsigned long long)kProbe)
+    if (time_bound<MODE, false>(a.prog[pc.prog], a.prm, cwait) >= (unsigned long long)kProbe)
       atomicExch(a.pcs.fail + pc.split, 1);
   }
   bool bad = false;
@@ -78,35 +76,16 @@ __device__ __forceinline__ int32_t start_cursor(const SweepArgs& a, const SplitP
 // Slot of state variable v (cursor v < ne, last retire v - ne) in a 64-entry state.
 __device__ __forceinline__ int slot_of(int v, int ne) { return v < ne ? v : 32 + v - ne; }
 
-// One warp per split program: the pieces' start states in order, the
-// program's makespan and status; the checksum is zeroed for the fix-up pass
-// to accumulate.  Barrier scheme: every piece runs from a release, so it is
-// shifted by its start (stored in shift).  Barrier-free, probed programs:
-// the probes' end states give each piece's max-plus map (x at 64 * piece).
-template <bool BB>
+// One warp per probed program: the pieces' start states in order from the
+// probes' end states (x at 64 * piece), the program's makespan and status;
+// the checksum is zeroed for the fix-up pass to accumulate.
 __global__ void k_piece_resolve(const SweepArgs a, int n_split) {
   const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (w >= n_split) return;
   if (*(volatile int32_t*)(a.pcs.fail + w)) return;
-  if (!BB && a.pcs.cls[w]) return;                 // speculated, not probed
+  if (a.pcs.cls[w]) return;                        // speculated, not probed
   const SplitProg sp = a.pcs.split[w];
   const int ne = sp.ne;
-  if (BB) {
-    // after L's statement barrier every engine is at c_barrier; each piece
-    // ends with a barrier release, its duration after its start
-    int64_t R = a.prm.c_barrier;
-    for (int j = 0; j < sp.n_pieces; ++j) {
-      const int piece = sp.first_piece + j;
-      if (lane == 0) a.pcs.shift[piece] = (int32_t)R;
-      R += __ldg(a.pcs.out + (int64_t)piece * a.pcs.out_probes * 64);   // run 0, engine 0: the release
-    }
-    if (lane == 0) {
-      a.makespan[sp.prog] = (int32_t)R;
-      a.status[sp.prog] = SYNC_PROG_OK;
-      a.checksum[sp.prog] = 0ull;
-    }
-    return;
-  }
   const int nv = 2 * ne;
   // lane holds variables lane and lane + 32
   int64_t x0 = lane < ne ? start_cursor(a, sp) : 0, x1 = 0;
@@ -254,10 +233,9 @@ __global__ void k_spec_resolve(const SweepArgs a, int n_split, int last_round) {
 // program; every instance of the piece gets its true issue and retire times
 // from the stored ones (see the top of this file) and adds its checksum
 // term; the timelines, if requested, are written here.  Stored times of
-// single runs (barrier scheme, speculated pieces) are in `one` (issue,
+// single runs (speculated pieces) are in `one` (issue,
 // retire, position in the engine's stream per instance of the split
 // programs, one_len of them), those of the probes in a.pcs.ptimes.
-template <bool BB>
 __global__ void __launch_bounds__(kValThreads) k_piece_fixup(const SweepArgs a, const int32_t* __restrict__ cnt,
                                                              const int32_t* __restrict__ one, int64_t one_len) {
   __shared__ int32_t xs[64];
@@ -266,7 +244,7 @@ __global__ void __launch_bounds__(kValThreads) k_piece_fixup(const SweepArgs a, 
   const PieceInfo pc = a.pcs.piece[piece];
   if (*(volatile int32_t*)(a.pcs.fail + pc.split)) return;
   const SplitProg sp = a.pcs.split[pc.split];
-  const bool shifted = BB || a.pcs.cls[pc.split];
+  const bool shifted = a.pcs.cls[pc.split];
   const int j = piece - sp.first_piece, ne = sp.ne, nv = 2 * ne;
   if (threadIdx.x < 64) xs[threadIdx.x] = shifted ? 0 : a.pcs.x[(int64_t)piece * 64 + threadIdx.x];
   __syncthreads();
@@ -333,27 +311,26 @@ cudaError_t launch_items(K kern, const SweepArgs& a, int64_t items, size_t smem,
   return launched();
 }
 
-template <int MODE, bool BB>
+template <int MODE>
 cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaStream_t s) {
   const size_t smem = sweep_smem_bytes(a.sem_cap, a.frame_depth, a.ring);
   const int warp_blocks = (L.n_split * 32 + 255) / 256;
-  k_piece_validate<MODE, BB><<<a.pcs.n_pieces, kValThreads, 0, s>>>(a, L.vdep, L.cnt);
+  k_piece_validate<MODE><<<a.pcs.n_pieces, kValThreads, 0, s>>>(a, L.vdep, L.cnt);
   cudaError_t e = launched();
   if (e != cudaSuccess) return e;
-  // barrier scheme, or barrier-free probes: one launch of runs storing
-  // every instance's times, then the composition
-  if (BB || L.n_probed > 0) {
+  // probes: one launch of runs storing every instance's times, then the
+  // composition
+  if (L.n_probed > 0) {
     SweepArgs p = a;
     p.pcs.spec = 0;
-    if (BB) { p.pcs.ptimes = L.one; p.pcs.plen = L.one_len; }
-    e = launch_items(k_sweep<MODE, BB, true, false, true>, p, (int64_t)p.pcs.n_pieces * p.pcs.probes, smem,
+    e = launch_items(k_sweep<MODE, false, true, false, true>, p, (int64_t)p.pcs.n_pieces * p.pcs.probes, smem,
                      num_sms, s);
     if (e != cudaSuccess) return e;
-    k_piece_resolve<BB><<<warp_blocks, 256, 0, s>>>(p, L.n_split);
+    k_piece_resolve<<<warp_blocks, 256, 0, s>>>(p, L.n_split);
     if ((e = launched()) != cudaSuccess) return e;
   }
-  // barrier-free speculation: rounds of runs and acceptance checks
-  if (!BB && L.n_spec > 0) {
+  // speculation: rounds of runs and acceptance checks
+  if (L.n_spec > 0) {
     SweepArgs p = a;
     p.pcs.spec = 1;
     p.pcs.probes = 1;
@@ -362,7 +339,7 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
     k_spec_init<<<warp_blocks, 256, 0, s>>>(p, L.n_split);
     if ((e = launched()) != cudaSuccess) return e;
     for (int r = 0; r < kSpecRounds; ++r) {
-      e = launch_items(k_sweep<MODE, BB, true, false, true>, p, p.pcs.n_pieces, smem, num_sms, s);
+      e = launch_items(k_sweep<MODE, false, true, false, true>, p, p.pcs.n_pieces, smem, num_sms, s);
       if (e != cudaSuccess) return e;
       k_spec_resolve<<<warp_blocks, 256, 0, s>>>(p, L.n_split, r == kSpecRounds - 1);
       if ((e = launched()) != cudaSuccess) return e;
@@ -370,20 +347,17 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
   }
   // (piece, instruction slice) blocks: about 2048 or more in all
   const int ys = std::max(1, std::min(a.pcs.nx_max, (2048 + a.pcs.n_pieces - 1) / a.pcs.n_pieces));
-  k_piece_fixup<BB><<<dim3(a.pcs.n_pieces, ys), kValThreads, 0, s>>>(a, L.cnt, L.one, L.one_len);
+  k_piece_fixup<<<dim3(a.pcs.n_pieces, ys), kValThreads, 0, s>>>(a, L.cnt, L.one, L.one_len);
   return launched();
 }
 
 }  // namespace
 
-cudaError_t launch_pieces(const SweepArgs& a, bool barrier, const PieceLaunch& L, int num_sms, cudaStream_t s) {
+cudaError_t launch_pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaStream_t s) {
   if (a.pcs.n_pieces == 0 || L.n_split == 0) return cudaSuccess;
-  if (a.mode == SYNC_THR_PERLOOP)
-    return barrier ? pieces<SYNC_THR_PERLOOP, true>(a, L, num_sms, s) : pieces<SYNC_THR_PERLOOP, false>(a, L, num_sms, s);
-  if (a.mode == SYNC_THR_PERENGINE)
-    return barrier ? pieces<SYNC_THR_PERENGINE, true>(a, L, num_sms, s)
-                   : pieces<SYNC_THR_PERENGINE, false>(a, L, num_sms, s);
-  return barrier ? pieces<SYNC_THR_COUNT, true>(a, L, num_sms, s) : pieces<SYNC_THR_COUNT, false>(a, L, num_sms, s);
+  if (a.mode == SYNC_THR_PERLOOP) return pieces<SYNC_THR_PERLOOP>(a, L, num_sms, s);
+  if (a.mode == SYNC_THR_PERENGINE) return pieces<SYNC_THR_PERENGINE>(a, L, num_sms, s);
+  return pieces<SYNC_THR_COUNT>(a, L, num_sms, s);
 }
 
 }  // namespace syncgb

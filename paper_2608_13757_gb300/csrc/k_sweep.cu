@@ -14,15 +14,19 @@ cudaError_t launch3(const SweepArgs& a, size_t smem, int num_sms, cudaStream_t s
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const long long want = ((long long)a.n_programs + kWarps - 1) / kWarps;
+    const long long items = a.bar.on && a.bar.n_tiles > a.n_programs ? a.bar.n_tiles : a.n_programs;
+    const long long want = (items + kWarps - 1) / kWarps;
     const long long cap = (long long)num_sms * per_sm;
     const int grid = (int)(want < cap ? want : cap);
-    e = cudaMemsetAsync(a.next_slot, 0, sizeof(int32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.fallback, 0, sizeof(int32_t), s);
+    // the launch's counters: next_slot up to fallback[0]
+    e = cudaMemsetAsync(a.next_slot, 0, (size_t)(a.fallback + 1 - a.next_slot) * sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
     kern<<<grid, kWarps * 32, smem, s>>>(a);
     return launched();
   };
+  if constexpr (BB)
+    if (a.bar.on || a.bar.todo)
+      return a.issue ? run(k_sweep<MODE, true, true, false, false, true>) : run(k_sweep<MODE, true, false, false, false, true>);
   if (a.dep) return a.issue ? run(k_sweep<MODE, BB, true, true>) : run(k_sweep<MODE, BB, false, true>);
   return a.issue ? run(k_sweep<MODE, BB, true, false>) : run(k_sweep<MODE, BB, false, false>);
 }

@@ -1,4 +1,4 @@
-// Tile tables of the threshold and derive kernels, built by the loader on
+// Tile tables of the threshold, derive and interval kernels, built by the loader on
 // the device from the tables it copied there.
 #include "progbuild.cuh"
 
@@ -36,6 +36,11 @@ struct JobRowStart {
   __device__ int64_t operator()(int64_t i) const { return jobs[i].row0; }
 };
 
+struct LoopTileStart {
+  const BarLoop* bl;
+  __device__ int64_t operator()(int64_t i) const { return bl[i].tile0; }
+};
+
 int grid_for(int64_t n, int threads, int num_sms) {
   const int64_t want = (n + threads - 1) / threads;
   const int64_t cap = (int64_t)num_sms * 16;
@@ -53,9 +58,12 @@ cudaError_t tile_table(int32_t* table, int64_t n_tiles, int64_t n, int64_t tile,
 
 cudaError_t launch_tile_tables(const int64_t* seg, int64_t n_deps, int32_t* tile_first, int64_t n_first_tiles,
                                const DeriveJob* jobs, int64_t n_jobs, int32_t* tile_job, int64_t n_job_tiles,
+                               const BarLoop* bl, int64_t n_loops, int32_t* tile_loop, int64_t n_tiles,
                                int num_sms, cudaStream_t s) {
   cudaError_t e = tile_table(tile_first, n_first_tiles, n_deps, kTilePairs, SegStart{seg}, num_sms, s);
   if (e == cudaSuccess) e = tile_table(tile_job, n_job_tiles, n_jobs, kJobTileRows, JobRowStart{jobs}, num_sms, s);
+  if (e == cudaSuccess && n_tiles > 0)
+    e = tile_table(tile_loop, n_tiles, n_loops, 1, LoopTileStart{bl}, num_sms, s);
   return e;
 }
 

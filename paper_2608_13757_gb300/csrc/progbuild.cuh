@@ -56,6 +56,8 @@ enum : int32_t {
   BC_SEMHB,        // semaphore history bases
   BC_JOBS,         // derive jobs
   BC_DROWS,        // rows of the derive jobs
+  BC_FPOOL,        // interval starts of inner loops (BarLoop)
+  BC_TILES,        // interval tiles
   kBuildCounts
 };
 
@@ -94,19 +96,20 @@ struct Seen {
 // dependency [ND], per (loop, engine) row [rows]; body items of program p
 // at x0 + l0 (nx + nl - 1 of them), body offsets at l0 + p (nl + 1).
 struct BuildScratch {
-  int32_t *depth, *lfill;                    // [NL]
-  uint8_t *needs_rhat, *fbar;                // [NL]
+  int32_t *depth, *lfill, *cidx;             // [NL]
+  uint8_t *needs_rhat, *fbar, *unit;         // [NL] (unit: 1 = every trip is 1, 2 = and so below it)
   int32_t* body_ptr;                         // [NL + P]
   int64_t* keys;                             // [NX + NL]
   int32_t* body;                             // [NX + NL]
-  int32_t *rank, *x_ndeps, *x_dep_begin, *x_levels, *cons_next, *sem_x;   // [NX]
-  int32_t *nloop_eng, *sem_row;              // [rows]
+  int32_t *rank, *x_ndeps, *x_dep_begin, *x_levels, *cons_next, *sem_x, *op_of, *prevc;   // [NX]
+  int32_t *nloop_eng, *sem_row, *fix_cnt, *before;   // [rows]
   int64_t *stot, *srp, *tstart;              // [rows] per iteration space
   uint32_t* pe_of;                           // [rows]
   uint8_t* rpflag;                           // [rows]
   int32_t* anc;                              // [rows * SYNC_MAX_DEPTH]
   uint8_t* dep_bar;                          // [ND]
-  int32_t *dep_S, *dep_N, *by_cons;          // [ND]
+  int32_t *dep_S, *dep_N, *by_cons, *dep_ca, *dep_cb;   // [ND] (ca, cb: S's children towards producer and consumer)
+  uint8_t* dep_fix;                          // [ND]: bit 0 / 1: only fixed loops from S to producer / consumer
   Seen* seen;                                // [ND]
 };
 
@@ -131,14 +134,15 @@ struct BuildOut {
   int32_t* op_ptr;         // [rows + 1]
   int2* rowinfo;           // [rows]
   int32_t* hoist;          // [rows]
-  LoopInfo* xloops;        // [NL] (shared trips) or [rows] (per-engine trips)
-  uint8_t* reads_rowptr;   // like xloops
   int32_t* rowptr;         // appended from here on
   int64_t* path;
   DeriveJob* jobs;
   int4 *ops, *plan, *paux, *chunks, *lrec, *lmeta;
   int32_t* opstop;
   int64_t* semhb;
+  BarLoop* bl;             // [NL + 1]
+  BarDep* bdep;            // [ND]
+  int2* rowc;              // [rows]
 };
 
 // What COUNT reports per program besides the counts.
@@ -211,7 +215,7 @@ struct ProgBuilder {
   const BuildScratch& S;
   const BuildOut& O;
   int32_t p, l0, x0, d0, nl, nx, nd, ne;
-  int64_t row0, xbase;
+  int64_t row0;
   const int32_t *par, *lpos;
   int64_t c[kBuildCounts];
   int64_t inst_eng[32];      // instances per engine
@@ -227,7 +231,6 @@ struct ProgBuilder {
     nd = d.prog_dep_ptr[p + 1] - d0;
     ne = d.prog_n_engines[p];
     row0 = d.row_base[p];
-    xbase = d.div ? row0 : l0;
     par = d.loop_parent + l0;
     lpos = d.loop_pos + l0;
     for (int i = 0; i < kBuildCounts; ++i) c[i] = FILL ? A.base[(int64_t)p * kBuildCounts + i] : 0;
@@ -246,7 +249,6 @@ struct ProgBuilder {
   // the loop's engine-0 row otherwise
   PB_HD int64_t sr(int32_t l, int32_t e) const { return row0 + (int64_t)l * ne + (d.div ? e : 0); }
   PB_HD int64_t tot(int32_t l, int32_t e) const { return S.stot[sr(l, e)]; }
-  PB_HD int32_t xid(int32_t l, int32_t e) const { return d.div ? l * ne + e : l; }
   PB_HD int32_t depth(int32_t l) const { return S.depth[l0 + l]; }
 
   // ------------------------------------------------------------ loops
@@ -280,10 +282,20 @@ struct ProgBuilder {
   // iteration), total and trip prefix sums
   PB_HD bool add_space(int32_t l, int32_t e, const int32_t* trips, int64_t want) {
     int64_t t = 0;
-    for (int64_t j = 0; j < want; ++j) {
-      if (trips[j] < 0) return fail(BE_TRIP_NEG, l);
-      t += trips[j];
+    if (FILL) {
+      t = S.stot[row0 + (int64_t)l * ne + e];
+    } else {
+      int32_t any = 0;                         // sign: some trip is negative
+      for (int64_t j = 0; j < want; ++j) {
+        any |= trips[j];
+        t += trips[j];
+      }
+      if (any < 0) return fail(BE_TRIP_NEG, l);
     }
+    // (t = want with no trip above 1: every trip is 1)
+    int32_t other = t != want;
+    for (int64_t j = 0; !FILL && !other && j < want; ++j) other = trips[j] != 1;
+    if (!FILL) S.unit[l0 + l] = !d.div && l > 0 && other == 0;
     if (l == 0 && t != 1) return fail(BE_TOP_TRIP, 0);
     if (t > kI32Max) return fail(BE_ITERS, l);
     const int64_t r = row0 + (int64_t)l * ne + e;
@@ -297,8 +309,6 @@ struct ProgBuilder {
       L.n_parent = (int32_t)want;
       L.depth = depth(l);
       L.rowptr_off = c[BC_ROWPTR];
-      const int64_t xi = xbase + xid(l, e);
-      O.xloops[xi] = L;
       int32_t* rp = O.rowptr + c[BC_ROWPTR];
       int32_t acc = 0;
       rp[0] = 0;
@@ -376,6 +386,24 @@ struct ProgBuilder {
       }
     }
     return true;
+  }
+
+  PB_HD bool fixed(int32_t l) const { return S.unit[l0 + l] == 2; }
+
+  // fixed loops (BarLoop in enc.h) and, per (loop, engine), the instances of
+  // one iteration with the fixed child loops'
+  PB_HD void fixed_loops() {
+    if (FILL) return;
+    for (int32_t l = 0; l < nl; ++l) S.unit[l0 + l] = S.unit[l0 + l] ? 2 : 0;
+    for (int64_t i = 0; i < (int64_t)nl * ne; ++i) S.fix_cnt[row0 + i] = S.nloop_eng[row0 + i];
+    for (int32_t l = nl - 1; l > 0; --l) {
+      if (!fixed(l)) {
+        S.unit[l0 + par[l]] = 0;
+        continue;
+      }
+      for (int32_t e = 0; e < ne; ++e)
+        S.fix_cnt[row0 + (int64_t)par[l] * ne + e] += S.fix_cnt[row0 + (int64_t)l * ne + e];
+    }
   }
 
   // N (instructions directly in a loop body on one engine) and K (rank)
@@ -458,12 +486,22 @@ struct ProgBuilder {
       if (off < 0) return fail(BE_D_OFFSET, k);
       const int32_t Pl = IL(px), Cl = IL(cx);
       // climb to the innermost common loop; remember the child of it on each side
-      int32_t a = Pl, b = Cl, ca = -1, cb = -1;
-      while (depth(a) > depth(b)) { ca = a; a = par[a]; }
-      while (depth(b) > depth(a)) { cb = b; b = par[b]; }
-      while (a != b) { ca = a; a = par[a]; cb = b; b = par[b]; }
-      const int32_t Sl = a;
-      S.dep_S[gd] = Sl;
+      // (kept for FILL)
+      if (!FILL) {
+        int32_t a = Pl, b = Cl, na = -1, nb = -1;
+        bool fa = true, fb = true;
+        while (depth(a) > depth(b)) { na = a; fa = fa && fixed(a); a = par[a]; }
+        while (depth(b) > depth(a)) { nb = b; fb = fb && fixed(b); b = par[b]; }
+        while (a != b) {
+          na = a; fa = fa && fixed(a); a = par[a];
+          nb = b; fb = fb && fixed(b); b = par[b];
+        }
+        S.dep_S[gd] = a;
+        S.dep_ca[gd] = na;
+        S.dep_cb[gd] = nb;
+        S.dep_fix[gd] = (uint8_t)((fa ? 1 : 0) | (fb ? 2 : 0));
+      }
+      const int32_t Sl = S.dep_S[gd], ca = S.dep_ca[gd], cb = S.dep_cb[gd];
       const int32_t ppos = ca < 0 ? d.instr_pos[x0 + px] : lpos[ca];
       const int32_t cpos = cb < 0 ? d.instr_pos[x0 + cx] : lpos[cb];
       const bool forward = cpos > ppos;
@@ -776,6 +814,57 @@ struct ProgBuilder {
     }
   }
 
+  // a loop's interval starts and tiles (shared trips only)
+  PB_HD void bar_loop(int32_t l, int32_t nchild, int32_t nrec) {
+    const int64_t t = d.div ? 0 : tot(l, 0);
+    const int32_t iters = bar_iters(nrec, nchild);
+    if (FILL) {
+      BarLoop& b = O.bl[l0 + l];
+      b.foff = nchild > 0 ? c[BC_FPOOL] : -1;
+      b.prog = p;
+      b.nchild = nchild;
+      b.tile0 = (int32_t)c[BC_TILES];
+      b.iters = iters;
+    }
+    if (d.div) return;
+    if (nchild > 0) c[BC_FPOOL] += (1 + (int64_t)ne) * (2 * t + 1);
+    if (nrec > 0) c[BC_TILES] += (t + iters - 1) / iters;
+  }
+
+  // per waited dependency, the increments published at its consumer's
+  // interval (BarDep in enc.h)
+  PB_HD void bar_deps(int32_t nw) {
+    pi.nloops = nl;
+    pi.dep0 = d0;
+    pi.ndep = nw;
+    if (!FILL) return;
+    for (int32_t i = 0; i < nw; ++i) {
+      const int32_t k = S.by_cons[d0 + i];
+      const int32_t px = d.dep_prod[d0 + k], cx = d.dep_cons[d0 + k], ep = IE(px);
+      const int32_t ca = S.dep_ca[d0 + k], cb = S.dep_cb[d0 + k];
+      const int32_t pc = S.prevc[x0 + cx];        // the child loop before the consumer's segment
+      auto before = [&](int32_t m) { return m < 0 ? 0 : S.before[row0 + (int64_t)m * ne + ep]; };
+      BarDep b{};
+      b.prod_op = -1;
+      b.prod_fixed = S.dep_fix[d0 + k] & 1;
+      b.cons_fixed = S.dep_fix[d0 + k] >> 1;
+      b.ep = (uint8_t)ep;
+      b.b2 = before(pc);
+      b.cons_loop = l0 + IL(cx);
+      b.cons_item = pc < 0 ? -1 : O.bl[l0 + pc].item;
+      if (ca < 0) {
+        b.b[1] = before(cb < 0 ? pc : cb);
+        b.b[0] = S.rank[x0 + px] <= b.b[1] ? 1 : 0;
+        if (cb < 0 && S.prevc[x0 + px] == pc) b.prod_op = S.op_of[x0 + px];
+      } else if (cb < 0) {
+        b.delta = pc >= 0 && S.cidx[l0 + ca] <= S.cidx[l0 + pc] ? 1 : 0;
+      } else {
+        b.delta = S.cidx[l0 + ca] < S.cidx[l0 + cb] ? 1 : 0;
+      }
+      O.bdep[d0 + i] = b;
+    }
+  }
+
   // per-(loop, engine) op records: own instructions and child loops in body
   // order, then an END record; the next LOOP or END record at or after each
   PB_HD void op_rows() {
@@ -785,8 +874,13 @@ struct ProgBuilder {
       // every instruction on its engine's row, every child loop and an END
       // record on each engine's row
       for (int32_t l = 0; l < nl; ++l) {
-        int32_t nloops = 0;
-        for (int32_t i = bp[l]; i < bp[l + 1]; ++i) nloops += bd[i] < 0 ? 1 : 0;
+        int32_t nloops = 0, moving = 0;
+        for (int32_t i = bp[l]; i < bp[l + 1]; ++i)
+          if (bd[i] < 0) {
+            ++nloops;
+            moving += fixed(-bd[i] - 1) ? 0 : 1;
+          }
+        bar_loop(l, moving, bp[l + 1] - bp[l] - nloops);
         c[BC_OPS] += (bp[l + 1] - bp[l] - nloops) + (int64_t)ne * (nloops + 1);
       }
       return;
@@ -796,10 +890,15 @@ struct ProgBuilder {
     // engine's); a LOOP or END record closes the instructions before it
     // (their op stop is that record)
     int64_t pos[32], pend[32];
-    int32_t cnt[32];
+    int32_t cnt[32], own[32], all[32];
+    O.bl[l0].item = O.bl[l0].esib = 0;
+    O.bl[l0].host = l0;
     for (int32_t l = 0; l < nl; ++l) {
-      int32_t nloops = 0;
-      for (int32_t e = 0; e < ne; ++e) cnt[e] = 0;
+      int32_t nloops = 0, last_child = -1, child = 0, moving = 0;
+      for (int32_t e = 0; e < ne; ++e) {
+        cnt[e] = own[e] = 0;
+        all[e] = fixed(l) ? O.rowc[row0 + (int64_t)l * ne + e].x : 0;   // instances so far in the host's iteration
+      }
       for (int32_t i = bp[l]; i < bp[l + 1]; ++i) {
         const int32_t it = bd[i];
         if (it < 0) ++nloops; else ++cnt[IE(it)];
@@ -807,6 +906,8 @@ struct ProgBuilder {
       int64_t at = c[BC_OPS];
       for (int32_t e = 0; e < ne; ++e) {
         O.op_ptr[row0 + (int64_t)l * ne + e] = (int32_t)at;
+        if (l == 0) O.rowc[row0 + e].x = 0;
+        O.rowc[row0 + (int64_t)l * ne + e].y = S.fix_cnt[row0 + (int64_t)l * ne + e];
         pos[e] = pend[e] = at;
         at += cnt[e] + nloops + 1;
       }
@@ -818,17 +919,31 @@ struct ProgBuilder {
         const int32_t it = bd[i];
         if (it < 0) {
           const int32_t m = -it - 1;
+          last_child = m;
+          S.cidx[l0 + m] = child++;
+          O.bl[l0 + m].esib = moving;
+          O.bl[l0 + m].host = fixed(m) ? O.bl[l0 + l].host : l0 + m;
+          moving += fixed(m) ? 0 : 1;
           for (int32_t e = 0; e < ne; ++e) {
+            const int64_t mr = row0 + (int64_t)m * ne + e;
+            S.before[mr] = own[e];
+            O.rowc[mr].x = all[e];
+            if (fixed(m)) all[e] += S.fix_cnt[mr];
             const int64_t rp = S.srp[sr(m, e)], q = pos[e]++;
             O.ops[q] = make_int4(OP_LOOP, (int32_t)(row0 + (int64_t)m * ne), (int32_t)(uint32_t)(rp & 0xffffffffu),
                                  (int32_t)(rp >> 32));
             close(e, q);
           }
         } else {
+          ++own[IE(it)];
+          ++all[IE(it)];
+          S.prevc[x0 + it] = last_child;
+          S.op_of[x0 + it] = (int32_t)pos[IE(it)];
           O.ops[pos[IE(it)]++] = make_int4(x0 + it, d.instr_latency[x0 + it], S.x_ndeps[x0 + it],
                                            S.x_dep_begin[x0 + it]);
         }
       }
+      bar_loop(l, moving, bp[l + 1] - bp[l] - nloops);
       const int32_t flags = (nloops > 0 ? 1 : 0) | (O.lflag[l0 + l] ? 2 : 0) | (S.fbar[l0 + l] ? 4 : 0);
       for (int32_t e = 0; e < ne; ++e) {
         const int64_t row = row0 + (int64_t)l * ne + e, q = pos[e];
@@ -914,6 +1029,7 @@ struct ProgBuilder {
         if (!at_end) {
           ++nloops;
           const int32_t m = -it - 1;
+          if (FILL) O.bl[l0 + m].item = (int32_t)c[BC_PLAN];
           add_item(make_int4(ITEM_LOOP, l0 + m, FILL ? O.lflag[l0 + m] : 0, 0));
         }
       }
@@ -1005,10 +1121,10 @@ struct ProgBuilder {
 
   // the rowptr spaces the threshold kernels read (nested producers' loops)
   PB_HD void reads() {
+    if (FILL) return;
     for (int32_t l = 0; l < nl; ++l)
       for (int32_t e = 0; e < (d.div ? ne : 1); ++e) {
         const int64_t r = row0 + (int64_t)l * ne + e;
-        if (FILL) O.reads_rowptr[xbase + xid(l, e)] = S.rpflag[r];
         if (S.rpflag[r]) sm.struct_bytes += 4 * ((l == 0 ? 1 : S.stot[sr(par[l], e)]) + 1);
       }
   }
@@ -1017,6 +1133,7 @@ struct ProgBuilder {
     bool ok = loops() && spaces() && instrs() && bodies();
     if (ok) {
       ranks();
+      fixed_loops();
       aggregates();
       ok = deps();
     }
@@ -1028,6 +1145,7 @@ struct ProgBuilder {
       op_rows();
       const int64_t plan_first = c[BC_PLAN];
       plan();
+      bar_deps(nw);
       loop_statements(plan_first);
       reads();
     }
@@ -1037,6 +1155,7 @@ struct ProgBuilder {
         O.seg[d.ND] = c[BC_PADDED];
         O.op_ptr[d.row_base[d.P]] = (int32_t)c[BC_OPS];
         O.plan_ptr[d.prog_loop_ptr[d.P]] = (int32_t)c[BC_PLAN];
+        O.bl[d.prog_loop_ptr[d.P]].tile0 = (int32_t)c[BC_TILES];
       }
     } else {
       for (int i = 0; i < kBuildCounts; ++i) A.count[(int64_t)p * kBuildCounts + i] = ok ? c[i] : 0;
@@ -1049,10 +1168,11 @@ struct ProgBuilder {
   }
 };
 
-// Tile tables (k_tiles.cu) of the threshold kernels (segment starts) and
-// the derive kernel (job rows).
+// Tile tables (k_tiles.cu) of the threshold kernels (segment starts), the
+// derive kernel (job rows) and the barrier scheme's intervals (loops).
 cudaError_t launch_tile_tables(const int64_t* seg, int64_t n_deps, int32_t* tile_first, int64_t n_first_tiles,
                                const DeriveJob* jobs, int64_t n_jobs, int32_t* tile_job, int64_t n_job_tiles,
+                               const BarLoop* bl, int64_t n_loops, int32_t* tile_loop, int64_t n_tiles,
                                int num_sms, cudaStream_t s);
 
 }  // namespace syncgb

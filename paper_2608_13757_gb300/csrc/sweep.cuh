@@ -32,7 +32,7 @@
 // lane of its run.
 #pragma once
 
-#include "cost.cuh"
+#include "bar.cuh"
 #include "waitval.cuh"
 
 namespace syncgb {
@@ -869,12 +869,14 @@ __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, c
   return 0;
 }
 
-// PIECE: the warp runs pieces of split programs (see PieceArgs) instead of
-// whole programs: item = piece * probes + probe; the walk starts inside the
-// body of the piece's loop L at its first iteration start and ends after
-// its last iteration (barrier scheme: after that iteration's barrier).
-template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false>
-__global__ void __launch_bounds__(kWarps * 32, 3) k_sweep(const SweepArgs a) {
+// PIECE (barrier-free): the warp runs pieces of split programs (see
+// PieceArgs) instead of whole programs: item = piece * probes + probe; the
+// walk starts inside the body of the piece's loop L at its first iteration
+// start and ends after its last iteration.
+// BAR (barrier scheme, array thresholds): programs by intervals (bar.cuh),
+// and by the walk only those the intervals leave.
+template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false, bool BAR = false>
+__global__ void __launch_bounds__(kWarps * 32, BAR ? kBarCtas : 3) k_sweep(const __grid_constant__ SweepArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   WarpSmem S;
@@ -912,15 +914,45 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_sweep(const SweepArgs a) {
   const int32_t ic_full = BB ? a.prm.c_branch : a.prm.c_branch + 2 * a.prm.c_regop;
   auto stmt_cost_of = [&](int32_t flag) { return elide && flag ? 0 : a.prm.c_regop; };
 
-  const int32_t n_items = PIECE ? a.pcs.n_pieces * a.pcs.probes : a.n_programs;
+  // BAR: the programs' plans, then the tiles of their intervals
+  bool tiles = false, planned = true;
+  int tile = blockIdx.x * kWarps + wib;
+
+  const int32_t n_items = PIECE ? a.pcs.n_pieces * a.pcs.probes : BAR && a.bar.todo ? *a.bar.todo : a.n_programs;
   for (;;) {
-    int slot = 0;
-    if (lane == 0) slot = atomicAdd(a.next_slot, 1);
-    slot = __shfl_sync(kFull, slot, 0);
-    if (slot >= n_items) break;
+    int slot = 0, left = -1;
+    if (!BAR || !tiles) {
+      if (lane == 0) slot = atomicAdd(a.next_slot, 1);
+      slot = __shfl_sync(kFull, slot, 0);
+      if (slot >= n_items) {
+        if (!BAR || !a.bar.on) break;
+        tiles = true;
+        planned = bar_planned(a, lane);
+        continue;
+      }
+      if (BAR && a.bar.on) {
+        const int q = __ldg(a.order + slot);
+        const bool ok = bar_plan<MODE>(a, q, S.nn, lane);
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) atomicAdd(a.bar.plans, 1);
+        if (ok) continue;
+        left = q;
+      }
+    } else {
+      if (tile >= a.bar.n_tiles) break;
+      if (planned) left = bar_tile<MODE, TL>(a, tile, S.nn, lane);
+      else if (lane == 0) a.status[a.bar.bl[a.bar.tile_loop[tile]].prog] = SYNC_PROG_ROUND_GUARD;
+      tile += gridDim.x * kWarps;
+      if (left < 0) continue;
+    }
     int piece = 0, probe = 0, p;
     PieceInfo pc;
-    if (PIECE) {
+    if (BAR && left >= 0) {
+      p = left;
+    } else if (BAR && a.bar.todo) {
+      p = a.bar.todo[1 + slot];
+    } else if (PIECE) {
       piece = slot / a.pcs.probes;
       probe = slot - piece * a.pcs.probes;
       pc = a.pcs.piece[piece];
@@ -928,7 +960,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_sweep(const SweepArgs a) {
     } else {
       p = __ldg(a.order + slot);
       // a split program simulated by its pieces in this call
-      if (a.pcs.prog_split) {
+      if (!BB && a.pcs.prog_split) {
         const int32_t sp_ = __ldg(a.pcs.prog_split + p);
         if (sp_ >= 0 && !*(volatile int32_t*)(a.pcs.fail + sp_)) continue;
       }
@@ -938,8 +970,8 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_sweep(const SweepArgs a) {
       // a failed validation, a probe past this program's state variables, a
       // program of the other barrier-free class, a speculative piece with no
       // run due
-      if (*(volatile int32_t*)(a.pcs.fail + pc.split) || probe >= (BB || a.pcs.spec ? 1 : 2 * pi.ne)) continue;
-      if (!BB && (__ldg(a.pcs.cls + pc.split) != 0) != (a.pcs.spec != 0)) continue;
+      if (*(volatile int32_t*)(a.pcs.fail + pc.split) || probe >= (a.pcs.spec ? 1 : 2 * pi.ne)) continue;
+      if ((__ldg(a.pcs.cls + pc.split) != 0) != (a.pcs.spec != 0)) continue;
       if (a.pcs.spec && !*(volatile int32_t*)(a.pcs.need + piece)) continue;
     }
     // the iteration-start cost of global loop `loop` on lane `lane`'s engine
@@ -965,9 +997,9 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_sweep(const SweepArgs a) {
       if (lane == 0) { a.makespan[p] = -1; a.checksum[p] = 0; a.status[p] = SYNC_PROG_OVERFLOW; }
       continue;
     }
-    // probe runs write a private history (each probe its own); the barrier
-    // scheme's and the speculated pieces' single runs write the real one
-    const bool probe_hist = PIECE && !BB && !a.pcs.spec;
+    // probe runs write a private history (each probe its own); the speculated
+    // pieces' single runs write the real one
+    const bool probe_hist = PIECE && !a.pcs.spec;
     for (int i = lane; i < pi.nsem[MODE]; i += 32) {
       S.semv[i] = PIECE ? __ldg(a.pcs.pub + pc.pub_off[MODE] + i) : 0;
       S.semhb[i] = __ldg(a.semhb + pi.semhb_off[MODE] + i);
@@ -976,16 +1008,16 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_sweep(const SweepArgs a) {
     }
     if (PIECE) {
       // the start state: probe `probe` raises state variable `probe` (cursors
-      // 0..ne-1, then last retires) by kProbe; the barrier scheme runs from
-      // a release at 0.  The instances' times go to the compact scratch.
-      int32_t t0 = !BB && lane == probe ? kProbe : 0, l0 = !BB && lane + pi.ne == probe ? kProbe : 0;
+      // 0..ne-1, then last retires) by kProbe.  The instances' times go to
+      // the compact scratch.
+      int32_t t0 = lane == probe ? kProbe : 0, l0 = lane + pi.ne == probe ? kProbe : 0;
       if (a.pcs.spec && lane < pi.ne) {              // a speculative piece: its guessed start
         t0 = a.pcs.xhat[(int64_t)piece * 64 + lane];
         l0 = a.pcs.xhat[(int64_t)piece * 64 + 32 + lane];
       }
       S.t[lane] = t0; S.lr[lane] = l0;
       S.nn[lane] = lane < pi.ne ? __ldg(a.pcs.pub + pc.nbase_off + lane) : 0;
-      if (lane == 0) { S.tlx[0] = pc.tl[BB || a.pcs.spec ? 0 : 1]; S.tlx[1] = probe; }
+      if (lane == 0) { S.tlx[0] = pc.tl[a.pcs.spec ? 0 : 1]; S.tlx[1] = probe; }
     } else {
       S.t[lane] = 0; S.lr[lane] = 0; S.nn[lane] = 0;
     }
@@ -1011,7 +1043,6 @@ __global__ void __launch_bounds__(kWarps * 32, 3) k_sweep(const SweepArgs a) {
         if (sp == 0) {
           if (!PIECE) break;                           // the top-level loop runs once
           // a piece: its loop's next iteration, or the end of the piece
-          if (BB) barrier_all(S, pi.ne, a.prm.c_barrier, lane);
           if (++g >= g_end) break;
           if (lane < pi.ne) S.t[lane] += iter_cost;
           __syncwarp();

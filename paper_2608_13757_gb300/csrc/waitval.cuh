@@ -13,9 +13,13 @@ namespace syncgb {
 // Iterations of P that start inside the first x iterations of S (x may equal
 // total(S)): compose the trip prefix sums from S's child down to P.
 template <class A>
-__device__ __forceinline__ int32_t count_down(const A& a, const DepInfo& D, int32_t x) {
-  for (int i = 0; i < D.clen; ++i) x = __ldg(a.rowptr + __ldg(a.path + D.path + D.up + i) + x);
+__device__ __forceinline__ int32_t count_down(const A& a, const DepInfo& D, int32_t x, const int32_t* rowptr) {
+  for (int i = 0; i < D.clen; ++i) x = __ldg(rowptr + __ldg(a.path + D.path + D.up + i) + x);
   return x;
+}
+template <class A>
+__device__ __forceinline__ int32_t count_down(const A& a, const DepInfo& D, int32_t x) {
+  return count_down(a, D, x, a.rowptr);
 }
 
 template <class A>

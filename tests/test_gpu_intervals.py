@@ -1,0 +1,98 @@
+"""Barrier scheme by intervals (csrc/bar.cuh) against the oracle, at the sizes
+where its tiles and row searches can go wrong: trip totals around a lane, a
+warp and a tile, rows without iterations, bodies of more records than lanes,
+loops that run exactly once, moving loops beside each other, and thresholds
+that do not repeat, which send the program to the walk."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from tests.test_gpu_parity import ALL_MODES, compare_all
+
+pytestmark = pytest.mark.gpu
+
+PRM = dict(ii=2, c_branch=3, c_regop=2, c_barrier=9)
+
+
+@pytest.fixture(scope="module")
+def sg():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_13757_gb300 import build
+    build.build()
+    import paper_2608_13757_gb300 as m
+    return m
+
+
+def trips_of(total, rows, empty, rng):
+    """`rows` trips that add up to `total`, a share `empty` of them 0."""
+    t = np.zeros(rows, dtype=np.int64)
+    live = np.flatnonzero(rng.random(rows) >= empty)
+    if live.size == 0:
+        live = np.array([rows - 1])
+    np.add.at(t, rng.choice(live, size=total), 1)
+    return t.tolist()
+
+
+def program(total, rows, records, empty, rng):
+    """An outer loop of `rows` iterations around a leaf of `total`, with a
+    conditional taken always, one taken at times and a second moving loop."""
+    b = workloads.ProgramBuilder(3)
+    lat = lambda: int(rng.integers(1, 40))
+    A = b.loop(0, 1, [rows])
+    first = b.instr(0, 0, 0, lat())
+    a0 = b.instr(A, 0, 1, lat())
+    L = b.loop(A, 1, trips_of(total, rows, empty, rng))
+    once = b.loop(A, 2, [1] * rows)
+    inner = b.loop(once, 1, [1] * rows)
+    x0, x1, x2 = b.instr(once, 0, 2, lat()), b.instr(inner, 0, 0, lat()), b.instr(once, 2, 1, lat())
+    M = b.loop(A, 3, rng.integers(0, 3, size=rows).tolist())
+    c = b.loop(A, 4, rng.integers(0, 2, size=rows).tolist())
+    y, z, w = b.instr(M, 0, 2, lat()), b.instr(c, 0, 0, lat()), b.instr(A, 5, 1, lat())
+    xs = [b.instr(L, i, int(rng.integers(0, 3)), lat()) for i in range(records)]
+    for i in range(1, records):
+        if rng.random() < 0.5:
+            b.dep(xs[int(rng.integers(0, i))], xs[i], 0)
+        if rng.random() < 0.3:
+            b.dep(xs[int(rng.integers(i, records))], xs[i], 1 + int(rng.integers(0, 2)))
+    for p, q, k in ((first, xs[0], 0), (a0, xs[-1], 0), (x0, x1, 0), (x1, x2, 0), (x2, x0, 1), (xs[0], x1, 0),
+                    (x1, y, 0), (y, z, 0), (z, w, 0), (w, a0, 1), (xs[-1], a0, 1), (y, xs[0], 1)):
+        b.dep(p, q, k)
+    return b.batch()
+
+
+@pytest.mark.parametrize("rows,empty", [(1, 0.0), (5, 0.0), (90, 0.6)])
+def test_tile_edges(sg, rows, empty):
+    rng = np.random.default_rng(rows)
+    parts = [program(total, rows, records, empty, rng)
+             for total in (0, 1, 31, 32, 33, 127, 128, 129, 385, 513) for records in (1, 3, 17, 33, 66)]
+    compare_all(sg, workloads.concat(parts), timeline=True, modes=ALL_MODES, params=oracle.sim_params(**PRM))
+
+
+@pytest.mark.parametrize("mode", [oracle.COUNT, oracle.PERLOOP])
+def test_waits_that_do_not_repeat(sg, mode):
+    """Single thresholds moved to earlier increments, to none and past the
+    end: the walk's results, deadlocks among them."""
+    import torch
+    rng = np.random.default_rng(11)
+    batch = workloads.concat([program(129, 7, 9, 0.2, rng) for _ in range(12)])
+    h = sg.sync_load_programs(batch)
+    want = oracle.thresholds(batch, mode).copy()
+    own = np.repeat(np.arange(batch.n_deps), h.pair_counts)
+    prog = np.searchsorted(batch.prog_dep_ptr, own, side="right") - 1
+    for p in range(0, 11):
+        at = np.flatnonzero((prog == p) & (want > 0))
+        want[rng.choice(at)] += (-1, 1, -want[at].max(), 10 ** 6)[p % 4] if p < 8 else 0
+    want = np.maximum(want, 0)
+    thr = sg.sync_eval_thresholds(h, mode)
+    thr[torch.from_numpy(h.unpadded_index()).to(thr.device)] = torch.from_numpy(want).to(thr.device)
+    ref = oracle.simulate(batch, want, mode, oracle.BARRIER)
+    r = sg.sync_simulate(h, mode, thr, variant=oracle.BARRIER)
+    P = batch.n_programs
+    assert np.array_equal(r.status.cpu().numpy()[:P], ref.status)
+    assert np.array_equal(r.makespan.cpu().numpy()[:P], ref.makespan)
+    assert np.array_equal(r.checksum.cpu().numpy()[:P].view(np.uint64), ref.checksum)
+    assert (ref.status == 0).any() and (ref.status != 0).any()
+    h.close()
