@@ -840,6 +840,7 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
     code_unrolled += s.code_unrolled;
     n_bar_deps += s.n_bar_deps;
     h.max_inst = std::max(h.max_inst, s.n_inst);
+    h.n_stmt += s.n_stmt;
     ne_max = std::max(ne_max, s.ne);
     depth_max = std::max(depth_max, s.depth_max);
     ord_overflow |= s.ord_overflow;
@@ -1124,7 +1125,9 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
     a.dep = h->dep; a.ddep = h->ddep; a.path = h->path; a.ord = h->ord;
     a.chk_counts = d_counts; a.chk_first = reinterpret_cast<unsigned long long*>(d_first_bad);
   }
-  const int ring = sweep_ring_for(a.sem_cap, a.frame_depth, 200 * 1024);
+  const bool maps = variant != SYNC_SIM_BARRIER &&
+                    sweep_maps(h->sz.n_programs, h->sz.n_instances, h->n_stmt, h->num_sms);
+  const int ring = sweep_ring(a.sem_cap, a.frame_depth, maps);
   if (simulate_smem_bytes(a.warps, a.sem_cap, a.frame_depth) > 200 * 1024 || ring == 0)
     raise(SYNC_ERR_ARG, "a program has too many waited semaphores for the simulator's shared memory");
   SweepArgs w;
@@ -1141,12 +1144,14 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
   w.cost = h->cost;
   w.dep = a.dep; w.ddep = a.ddep; w.path = a.path; w.ord = a.ord;
   w.chk_counts = a.chk_counts; w.chk_first = a.chk_first;
+  w.maps = maps;
+  if (variant != SYNC_SIM_BARRIER && (maps || h->n_split > 0)) w.bar = h->bar;   // trip maps read the dependencies' tables
   const bool barrier = variant == SYNC_SIM_BARRIER;
   // barrier scheme (array thresholds): by intervals, in the sweep's launch or,
   // with split programs, in launches of its own
   if (!fused && barrier && h->bar.on && h->max_inst >= kBarMinInst) {
     w.bar = h->bar;
-    if (const int r = sweep_ring_for(a.sem_cap, a.frame_depth, kBarRingBytes)) w.ring = r;
+    if (const int r = sweep_ring_for(a.sem_cap, a.frame_depth, false, kBarRingBytes)) w.ring = r;
     w.bar.min_inst = kBarMinInst;
     if (h->n_split > 0) {
       cuda_check(launch_intervals(w, h->todo, h->sz.n_loops, st), "interval simulation");

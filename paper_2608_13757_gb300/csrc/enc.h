@@ -446,6 +446,7 @@ struct SweepArgs {
   CostTables cost;
   PieceArgs pcs;             // piece-parallel simulation (prog_split NULL: none)
   BarArgs bar;               // barrier scheme by intervals
+  int32_t maps;              // barrier-free: leaf trips by their maps (trip.cuh)
 };
 
 // Launchers (return the launch error, if any).
@@ -475,7 +476,18 @@ cudaError_t launch_simulate(const SimArgs& a, bool barrier, int num_sms, cudaStr
 // forward in program order are listed in a.fallback and then simulated by
 // the per-engine kernel (launch_simulate with SimArgs::only set).
 cudaError_t launch_sweep(const SweepArgs& a, bool barrier, int num_sms, cudaStream_t s);
-size_t sweep_smem_bytes(int sem_cap, int frame_depth, int ring);
+size_t sweep_smem_bytes(int sem_cap, int frame_depth, int ring, bool maps);
+cudaError_t launch_sweep_maps(const SweepArgs& a, int num_sms, cudaStream_t s);
+// Whether the barrier-free sweep of a batch takes its leaf loops' trips by
+// their maps (trip.cuh; 16 warps per SM instead of 24): where the longest
+// programs bound it, and where trips hold most of the work.  Chain programs
+// (264 instances per loop statement), walked / by maps: 4864 12.7 / 8.0 ms,
+// 8192 12.9 / 9.5, 16384 14.5 / 14.6, 32768 16.4 / 21.3; depth2 (540)
+// 16384 6.9 / 4.5, attention (393) 500 94 / 29; branching trees (7) 6000
+// 0.86 / 1.24, conditionals around one instruction (1) 2432 17.0 / 20.2.
+inline bool sweep_maps(int32_t n_programs, int64_t n_instances, int64_t n_statements, int num_sms) {
+  return n_instances >= 32 * n_statements && (n_programs <= 80 * num_sms || n_instances >= 320 * n_statements);
+}
 // Piece-parallel simulation of the split programs (a.pcs), barrier-free:
 // validation, the probe runs or speculation, the composition of the pieces, and the pass that forms the instances' true times (checksums,
 // timelines); the programs it completes are marked in a.pcs.fail (0) for
@@ -493,8 +505,10 @@ cudaError_t launch_pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms,
 // cannot do are listed in todo for launch_sweep.
 cudaError_t launch_intervals(const SweepArgs& a, int32_t* todo, int32_t n_loops, cudaStream_t s);
 // Largest ring (32, 16, ..., 1) whose sweep shared memory fits in `limit`
-// bytes, or 0 if none does.
-int sweep_ring_for(int sem_cap, int frame_depth, size_t limit);
+// bytes, or 0 if none does; and the sweep's own choice: with maps 80 KB a
+// CTA, two of which share an SM, else what one CTA may have.
+int sweep_ring_for(int sem_cap, int frame_depth, bool maps, size_t limit);
+int sweep_ring(int sem_cap, int frame_depth, bool maps);
 size_t simulate_smem_bytes(int warps, int sem_cap, int frame_depth);
 
 // Kernels this library has launched in this process (every handle and

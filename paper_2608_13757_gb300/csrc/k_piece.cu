@@ -313,7 +313,6 @@ cudaError_t launch_items(K kern, const SweepArgs& a, int64_t items, size_t smem,
 
 template <int MODE>
 cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaStream_t s) {
-  const size_t smem = sweep_smem_bytes(a.sem_cap, a.frame_depth, a.ring);
   const int warp_blocks = (L.n_split * 32 + 255) / 256;
   k_piece_validate<MODE><<<a.pcs.n_pieces, kValThreads, 0, s>>>(a, L.vdep, L.cnt);
   cudaError_t e = launched();
@@ -323,6 +322,8 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
   if (L.n_probed > 0) {
     SweepArgs p = a;
     p.pcs.spec = 0;
+    p.ring = sweep_ring(p.sem_cap, p.frame_depth, false);
+    const size_t smem = sweep_smem_bytes(p.sem_cap, p.frame_depth, p.ring, false);
     e = launch_items(k_sweep<MODE, false, true, false, true>, p, (int64_t)p.pcs.n_pieces * p.pcs.probes, smem,
                      num_sms, s);
     if (e != cudaSuccess) return e;
@@ -333,13 +334,15 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
   if (L.n_spec > 0) {
     SweepArgs p = a;
     p.pcs.spec = 1;
+    p.ring = sweep_ring(p.sem_cap, p.frame_depth, true);
+    const size_t smem = sweep_smem_bytes(p.sem_cap, p.frame_depth, p.ring, true);
     p.pcs.probes = 1;
     p.pcs.ptimes = L.one;
     p.pcs.plen = L.one_len;
     k_spec_init<<<warp_blocks, 256, 0, s>>>(p, L.n_split);
     if ((e = launched()) != cudaSuccess) return e;
     for (int r = 0; r < kSpecRounds; ++r) {
-      e = launch_items(k_sweep<MODE, false, true, false, true>, p, p.pcs.n_pieces, smem, num_sms, s);
+      e = launch_items(k_sweep<MODE, false, true, false, true, false, true>, p, p.pcs.n_pieces, smem, num_sms, s);
       if (e != cudaSuccess) return e;
       k_spec_resolve<<<warp_blocks, 256, 0, s>>>(p, L.n_split, r == kSpecRounds - 1);
       if ((e = launched()) != cudaSuccess) return e;

@@ -7,45 +7,38 @@ namespace {
 
 template <int MODE, bool BB>
 cudaError_t launch3(const SweepArgs& a, size_t smem, int num_sms, cudaStream_t s) {
-  auto run = [&](auto kern) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const long long items = a.bar.on && a.bar.n_tiles > a.n_programs ? a.bar.n_tiles : a.n_programs;
-    const long long want = (items + kWarps - 1) / kWarps;
-    const long long cap = (long long)num_sms * per_sm;
-    const int grid = (int)(want < cap ? want : cap);
-    // the launch's counters: next_slot up to fallback[0]
-    e = cudaMemsetAsync(a.next_slot, 0, (size_t)(a.fallback + 1 - a.next_slot) * sizeof(int32_t), s);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, kWarps * 32, smem, s>>>(a);
-    return launched();
-  };
-  if constexpr (BB)
+  long long items = a.n_programs;
+  auto run = [&](auto kern) { return run_sweep(kern, a, items, smem, num_sms, s); };
+  if constexpr (BB) {
+    if (a.bar.on && a.bar.n_tiles > items) items = a.bar.n_tiles;
     if (a.bar.on || a.bar.todo)
       return a.issue ? run(k_sweep<MODE, true, true, false, false, true>) : run(k_sweep<MODE, true, false, false, false, true>);
+  }
   if (a.dep) return a.issue ? run(k_sweep<MODE, BB, true, true>) : run(k_sweep<MODE, BB, false, true>);
   return a.issue ? run(k_sweep<MODE, BB, true, false>) : run(k_sweep<MODE, BB, false, false>);
 }
 
 }  // namespace
 
-size_t sweep_smem_bytes(int sem_cap, int frame_depth, int ring) {
-  return kWarps * warp_bytes(sem_cap, frame_depth, ring);
+size_t sweep_smem_bytes(int sem_cap, int frame_depth, int ring, bool maps) {
+  return kWarps * warp_bytes(sem_cap, frame_depth, ring, maps);
 }
 
-int sweep_ring_for(int sem_cap, int frame_depth, size_t limit) {
+int sweep_ring_for(int sem_cap, int frame_depth, bool maps, size_t limit) {
   for (int r = kRingMax; r >= 1; r >>= 1)
-    if (sweep_smem_bytes(sem_cap, frame_depth, r) <= limit) return r;
+    if (sweep_smem_bytes(sem_cap, frame_depth, r, maps) <= limit) return r;
   return 0;
+}
+
+int sweep_ring(int sem_cap, int frame_depth, bool maps) {
+  const int r = maps ? sweep_ring_for(sem_cap, frame_depth, maps, 108 * 1024) : 0;
+  return r ? r : sweep_ring_for(sem_cap, frame_depth, maps, 200 * 1024);
 }
 
 cudaError_t launch_sweep(const SweepArgs& a, bool barrier, int num_sms, cudaStream_t s) {
   if (a.n_programs == 0) return cudaSuccess;
-  const size_t smem = sweep_smem_bytes(a.sem_cap, a.frame_depth, a.ring);
+  if (a.maps) return launch_sweep_maps(a, num_sms, s);
+  const size_t smem = sweep_smem_bytes(a.sem_cap, a.frame_depth, a.ring, false);
   if (a.mode == SYNC_THR_PERLOOP)
     return barrier ? launch3<SYNC_THR_PERLOOP, true>(a, smem, num_sms, s)
                    : launch3<SYNC_THR_PERLOOP, false>(a, smem, num_sms, s);

@@ -148,7 +148,7 @@ struct BuildOut {
 // What COUNT reports per program besides the counts.
 struct alignas(16) ProgSummary {
   int64_t work;            // simulated work (the simulators' program order)
-  int64_t n_inst;
+  int64_t n_inst, n_stmt;
   int64_t code_looped, code_unrolled;   // static instructions (code-size proxy)
   int64_t n_bar_deps;      // barrier-fallback dependencies
   int64_t struct_bytes;    // path entries and rowptr spaces the threshold kernels read
@@ -1161,6 +1161,7 @@ struct ProgBuilder {
       for (int i = 0; i < kBuildCounts; ++i) A.count[(int64_t)p * kBuildCounts + i] = ok ? c[i] : 0;
       sm.ne = ne;
       sm.n_inst = pi.n_inst;
+      sm.n_stmt = pi.n_stmt;
       sm.work = pi.n_inst + pi.n_pairs + (pi.n_stmt + pi.n_iter) * pi.ne;
       sm.splittable = !d.div && pi.fb_iters == 0;
       A.sum[p] = sm;

@@ -39,7 +39,10 @@ namespace syncgb {
 namespace {
 
 constexpr int kWarps = 8;                   // programs (warps) per CTA
-constexpr int kMaxIntra = 4;                // in-chunk waits per lane before falling back
+// In-chunk waits per lane before the program goes to the per-engine kernel:
+// 12 of 5 bits each in one 64-bit register (4 in a register each sent one of
+// 4096 depth2 programs there, whose 10 ms were the whole batch's)
+constexpr int kMaxIntra = 12;
 constexpr int kMaxDeps = 2;                 // dependencies per lane held in registers
 constexpr int kRingMax = 32;                // most recent increments kept per semaphore
 constexpr unsigned kFull = 0xffffffffu;
@@ -48,10 +51,15 @@ constexpr int SIM_FALLBACK = 9;             // internal: handed to the per-engin
 
 struct Frame { int32_t loop, item, g, g_end; };
 
+// A leaf loop's trip map in shared memory, per warp (trip.cuh).
+constexpr int kTripCols = 24;               // inputs
+constexpr int kTripInts = 2 * 32 * kTripCols + 32 * (kTripCols + 1) + 64 + 4 * 32 + 8 * 32 + 16;
+
 // Shared memory of one warp (program), 16-byte aligned.
-__host__ __device__ __forceinline__ size_t warp_bytes(int sem_cap, int frame_depth, int ring) {
-  const size_t per = (size_t)(20 + 4 * ring + 32) * sem_cap + sizeof(Frame) * (size_t)frame_depth +
-                     8 * (size_t)(frame_depth + 1) + 3 * 8 + 8 + 3 * 4 * 32 + 16 + 8;
+__host__ __device__ __forceinline__ size_t warp_bytes(int sem_cap, int frame_depth, int ring, bool maps) {
+  const size_t per = (maps ? 4 * (size_t)kTripInts : 0) + (size_t)(20 + 4 * ring + 32) * sem_cap +
+                     sizeof(Frame) * (size_t)frame_depth + 8 * (size_t)(frame_depth + 1) + 3 * 8 + 8 + 3 * 4 * 32 +
+                     16 + 8;
   return (per + 15) & ~(size_t)15;
 }
 
@@ -78,6 +86,7 @@ __device__ __forceinline__ bool hoists(const SweepArgs& a) {
 }
 
 struct WarpSmem {
+  int32_t* map;        // [kTripInts] trip map
   int32_t* t;          // [32] engine cursors
   int32_t* lr;         // [32] engine last retire
   int32_t* nn;         // [32] engine datapath instances so far
@@ -202,7 +211,8 @@ __device__ __forceinline__ void set_groups(const WarpSmem& S, const LaneRec& L, 
 // the in-chunk increments its waits targeted.
 struct BbRep {
   bool on = false;
-  int32_t sig = 0, issue = 0, retire = 0, t = 0;
+  uint64_t sig = 0;
+  int32_t issue = 0, retire = 0, t = 0;
 };
 
 // Barrier-free, whole iterations of one loop through run_chunk: the lane's
@@ -235,7 +245,7 @@ __device__ __forceinline__ int run_chunk(const SweepArgs& a, const WarpSmem& S, 
   // waits: increments before this chunk from the ring (or, if older, the
   // history), increments inside it by lane
   int32_t known = kNeg;                        // satisfied before this chunk (kNeg: none)
-  int intra[kMaxIntra];
+  uint64_t intra = 0;                          // their producers' lanes, 5 bits each
   int n_intra = 0;
   bool fallback = false;
   auto wait_on = [&](int32_t Tj, int32_t s) {
@@ -250,10 +260,7 @@ __device__ __forceinline__ int run_chunk(const SweepArgs& a, const WarpSmem& S, 
     const unsigned m = S.tag[s] == ctag ? S.grp[s] : 0u;
     const int k = Tj - pub;
     if (k > __popc(m) || n_intra == kMaxIntra) { fallback = true; return; }
-    const int src = S.rank_lane[s * 32 + k - 1];
-#pragma unroll
-    for (int i = 0; i < kMaxIntra; ++i)
-      if (i == n_intra) intra[i] = src;         // static indices: intra stays in registers
+    intra |= (uint64_t)S.rank_lane[s * 32 + k - 1] << (5 * n_intra);
     ++n_intra;
   };
 #pragma unroll
@@ -263,6 +270,17 @@ __device__ __forceinline__ int run_chunk(const SweepArgs& a, const WarpSmem& S, 
     wait_on(FUSED ? fused_wait<MODE>(a, S, rec.w + j, gl, lc, lo_c) : __ldg(a.thr + __ldg(a.dseg + rec.w + j) + gl),
             __ldg(a.dsem + rec.w + j));
   if (__ballot_sync(kFull, fallback)) return SIM_FALLBACK;
+  const int deepest = (int)__reduce_max_sync(kFull, (unsigned)n_intra);
+  // the latest of the lane's in-chunk producers' values, kNeg without any
+  auto latest = [&](int32_t of) {
+    int32_t m = kNeg;
+    uint64_t t = intra;
+    for (int i = 0; i < deepest; ++i, t >>= 5) {
+      const int32_t v = __shfl_sync(kFull, of, (int)t & 31);
+      if (i < n_intra) m = max(m, v);
+    }
+    return m;
+  };
 
   const int32_t wcost = BB ? 0 : wait_ops<MODE>(a, rec, sr.w);
   // iter_cost is the iteration-start cost of lane `lane`'s engine (engines
@@ -277,15 +295,9 @@ __device__ __forceinline__ int run_chunk(const SweepArgs& a, const WarpSmem& S, 
   // relative to t_in depends only on which in-chunk increments the waits
   // target (their source lanes, 5 bits each, and their count): the same
   // targets as the last computed iteration give its schedule, shifted
-  int32_t sig = 0;
+  const uint64_t sig = (uint64_t)n_intra << 60 | intra;
   bool replay = false;
-  if (REP) {
-    sig = n_intra;
-#pragma unroll
-    for (int i = 0; i < kMaxIntra; ++i)
-      if (i < n_intra) sig |= intra[i] << (3 + 5 * i);
-    replay = rp.on && !__ballot_sync(kFull, valid && sig != rp.sig);
-  }
+  if (REP) replay = rp.on && !__ballot_sync(kFull, valid && sig != rp.sig);
   // PRED (barrier-free, whole iterations): extrapolate each lane's issue and
   // retire from the last two iterations and run one pass of the model on
   // it; if the pass reproduces the prediction on every lane, the prediction
@@ -295,13 +307,7 @@ __device__ __forceinline__ int run_chunk(const SweepArgs& a, const WarpSmem& S, 
   bool predicted = false;
   if (PRED && pd.n >= 2) {
     const int32_t pi_ = pd.issue + pd.d_issue, pr_ = pd.retire + pd.d_retire;
-    int32_t nr = kNeg;
-#pragma unroll
-    for (int i = 0; i < kMaxIntra; ++i) {
-      const int32_t src = i < n_intra ? intra[i] : lane;
-      const int32_t rv = __shfl_sync(kFull, pr_, src);
-      if (i < n_intra) nr = max(nr, rv);
-    }
+    const int32_t nr = latest(pr_);
     const int32_t ready = max(known, nr);
     int32_t Ai = A, Bi = (valid && ready >= 0) ? ready + a.prm.ii : kNeg;
 #pragma unroll
@@ -330,7 +336,7 @@ __device__ __forceinline__ int run_chunk(const SweepArgs& a, const WarpSmem& S, 
     t_after = t_in + rp.t;
   } else if (!predicted) {
   int32_t r_intra = kNeg;                      // retire of in-chunk producers (lower bound)
-  const bool any_intra = __ballot_sync(kFull, n_intra > 0) != 0;
+  const bool any_intra = deepest > 0;
   const int passes = any_intra ? ch.y + 2 : 1;
   bool settled = false;
   for (int pass = 0; pass < passes; ++pass) {
@@ -356,13 +362,7 @@ __device__ __forceinline__ int run_chunk(const SweepArgs& a, const WarpSmem& S, 
     if (!any_intra) { settled = true; break; }
     // new lower bound from the in-chunk producers' retire times; settled
     // once it binds nowhere (no issue would move)
-    int32_t nr = kNeg;
-#pragma unroll
-    for (int i = 0; i < kMaxIntra; ++i) {
-      const int32_t src = i < n_intra ? intra[i] : lane;
-      const int32_t rv = __shfl_sync(kFull, retire, src);
-      if (i < n_intra) nr = max(nr, rv);
-    }
+    const int32_t nr = latest(retire);
     if (!__ballot_sync(kFull, valid && nr > issue)) { settled = true; break; }
     r_intra = nr;
   }
@@ -390,8 +390,9 @@ __device__ __forceinline__ int run_chunk(const SweepArgs& a, const WarpSmem& S, 
   if (prod) {
     // the increment this retirement makes: per-engine semaphores count the
     // engine's instances, the others a fixed number per iteration
+    // (of a chunk's increments the ring keeps its own number, the last ones)
     const int32_t n = sr.y < 0 ? (int32_t)nj : sr.y * gl + sr.z;
-    S.ring[sr.x * (S.rmask + 1) + ((n - 1) & S.rmask)] = retire;
+    if (pub_own + __popc(S.grp[sr.x]) - n <= S.rmask) S.ring[sr.x * (S.rmask + 1) + ((n - 1) & S.rmask)] = retire;
     a.hist[S.semhb[sr.x] + (n - 1)] = retire;
   }
   if (valid) {
@@ -591,6 +592,7 @@ __device__ __forceinline__ int run_loop_regs(const SweepArgs& a, const WarpSmem&
         const int32_t cnt = present ? __popc(vm & my_run) : 0;   // engine `lane`'s instances per iteration
         const int32_t cnt_e = __shfl_sync(kFull, cnt, e), n_e = __shfl_sync(kFull, ns, e);
         const int32_t rank = __popc(vm & lanemask_le() & run_from_head);
+        const int32_t own_last = own_pub + J * __popc(own_grp & vm);
         if (have) {
           for (int32_t j = 0; j < J; ++j) {
             const int32_t bj = base + j * D, issue = bj + rd_issue, retire = bj + rd_retire;
@@ -598,7 +600,7 @@ __device__ __forceinline__ int run_loop_regs(const SweepArgs& a, const WarpSmem&
             const uint32_t nj = (uint32_t)(n_e + j * cnt_e + rank);
             if (prod_lane) {
               const int32_t n = own_stride < 0 ? (int32_t)nj : own_stride * gl + own_koff;
-              S.ring[own_ring + ((n - 1) & S.rmask)] = retire;
+              if (own_last - n <= S.rmask) S.ring[own_ring + ((n - 1) & S.rmask)] = retire;
               a.hist[own_hist + n] = retire;
             }
             chk += inst_term(issue, retire, (uint32_t)e, nj);
@@ -607,7 +609,7 @@ __device__ __forceinline__ int run_loop_regs(const SweepArgs& a, const WarpSmem&
         }
         pub0 += J * inc0;
         pub1 += J * inc1;
-        own_pub += J * __popc(own_grp & vm);
+        own_pub = own_last;
         const int32_t blast = base + (J - 1) * D;     // the run's last iteration
         if (lane < pi.ne) {
           if (present) {
@@ -735,9 +737,10 @@ __device__ __forceinline__ int run_loop_regs(const SweepArgs& a, const WarpSmem&
 
     // publish
     const uint32_t nj = (uint32_t)n_in + __popc(vm & lanemask_le() & run_from_head);
+    own_pub += __popc(own_grp & vm);
     if (valid && prod_lane) {
       const int32_t n = own_stride < 0 ? (int32_t)nj : own_stride * gl + own_koff;
-      S.ring[own_ring + ((n - 1) & S.rmask)] = retire;
+      if (own_pub - n <= S.rmask) S.ring[own_ring + ((n - 1) & S.rmask)] = retire;
       a.hist[own_hist + n] = retire;
     }
     if (valid) {
@@ -746,7 +749,6 @@ __device__ __forceinline__ int run_loop_regs(const SweepArgs& a, const WarpSmem&
     }
     pub0 += __popc(wg0 & vm);
     pub1 += __popc(wg1 & vm);
-    own_pub += __popc(own_grp & vm);
     if (present) {
       ts = t_last;
       lrs = r_last;
@@ -825,17 +827,29 @@ __device__ __forceinline__ int run_single(const SweepArgs& a, const WarpSmem& S,
   return 0;
 }
 
+}  // namespace
+}  // namespace syncgb
+
+#include "trip.cuh"
+
+namespace syncgb {
+namespace {
+
 // Iterations lo .. hi-1 of a loop whose body is one straight-line segment of
 // one chunk (or, barrier-free, one multi-iteration chunk); the first
 // iteration start has been charged.  The lane's record and thresholds stay
 // in registers; the next chunk's thresholds load while this one runs.
-// `one`: with a single iteration, the chunk holding its whole body
-// (zeros otherwise); a chunk of one record is applied directly.
-template <int MODE, bool BB, bool TL, bool FUSED>
+// `one`: the chunk holding one iteration's whole body; with a single
+// iteration of one record it is applied directly.
+template <int MODE, bool BB, bool TL, bool FUSED, bool MAPS>
 __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, const ProgInfo& pi, const int4 ch,
                                         const int4 one, int32_t lo, int32_t hi, int32_t ctag, int lane, int lc,
                                         int32_t iter_cost, unsigned long long& chk) {
-  if (one.y == 1) return run_single<MODE, BB, TL, FUSED>(a, S, pi, one, lo, lane, lc, chk);
+  if (hi - lo == 1 && one.y == 1) return run_single<MODE, BB, TL, FUSED>(a, S, pi, one, lo, lane, lc, chk);
+  if (MAPS && !FUSED) {
+    lo = run_trip<MODE, TL>(a, S, pi, one, lo, hi, lane, iter_cost, chk);
+    if (lo == hi) return 0;
+  }
   const int32_t copies = ch.z;
   const bool have = lane < ch.y;
   LaneRec L;
@@ -874,14 +888,17 @@ __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, c
 // walk starts inside the body of the piece's loop L at its first iteration
 // start and ends after its last iteration.
 // BAR (barrier scheme, array thresholds): programs by intervals (bar.cuh),
-// and by the walk only those the intervals leave.
-template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false, bool BAR = false>
-__global__ void __launch_bounds__(kWarps * 32, BAR ? kBarCtas : 3) k_sweep(const __grid_constant__ SweepArgs a) {
+// and by the walk only those the intervals leave.  MAPS (barrier-free): leaf
+// trips by their maps (trip.cuh).
+template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false, bool BAR = false, bool MAPS = false>
+__global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_sweep(const __grid_constant__ SweepArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   WarpSmem S;
   {
-    unsigned char* p = smem_raw + wib * warp_bytes(a.sem_cap, a.frame_depth, a.ring);
+    unsigned char* p = smem_raw + wib * warp_bytes(a.sem_cap, a.frame_depth, a.ring, MAPS);
+    S.map = reinterpret_cast<int32_t*>(p);
+    if (MAPS) p += 4 * kTripInts;
     // the walk-level table and check tallies go first in the barrier sweep and
     // last in the barrier-free one (a measured code-generation preference)
     S.semhb = reinterpret_cast<int64_t*>(p); p += 8 * a.sem_cap;
@@ -1021,6 +1038,13 @@ __global__ void __launch_bounds__(kWarps * 32, BAR ? kBarCtas : 3) k_sweep(const
     } else {
       S.t[lane] = 0; S.lr[lane] = 0; S.nn[lane] = 0;
     }
+    if (MAPS && lane == 0) {
+      // no trip map yet; maps add a time to a weight, both below 2^29 (probe
+      // runs raise times past that: none)
+      S.map[kTripHead] = -1;
+      S.map[kTripHead + 1] = 0;
+      S.map[kTripHead + 4] = a.bar.on && !(PIECE && !a.pcs.spec) && time_bound<MODE, BB>(pi, a.prm, cwait) < (1ull << 29);
+    }
     if (FUSED && lane == 0) {
       S.lvl[0] = make_int2(0, 0);                      // the top-level loop: iteration 0 of a trip at 0
       S.tally[0] = S.tally[1] = 0;
@@ -1090,7 +1114,7 @@ __global__ void __launch_bounds__(kWarps * 32, BAR ? kBarCtas : 3) k_sweep(const
           if (body_chunk >= 0) {
             // one iteration of one record: applied directly; otherwise a
             // loop around one chunk: all its iterations in registers
-            verdict = run_loop<MODE, BB, TL, FUSED>(a, S, pi, chb, hi - lo == 1 ? one : make_int4(0, 0, 0, 0), lo,
+            verdict = run_loop<MODE, BB, TL, FUSED, MAPS>(a, S, pi, chb, one, lo,
                                                     hi, ++ctag, lane, sp + 1, child_ic, chk);
             if (verdict) break;
             continue;
@@ -1190,6 +1214,25 @@ __global__ void __launch_bounds__(kWarps * 32, BAR ? kBarCtas : 3) k_sweep(const
     }
     __syncwarp();
   }
+}
+
+// Launches a sweep kernel with as many resident CTAs as its items take.
+template <class K>
+cudaError_t run_sweep(K kern, const SweepArgs& a, long long items, size_t smem, int num_sms, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, smem);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const long long want = (items + kWarps - 1) / kWarps;
+  const long long cap = (long long)num_sms * per_sm;
+  const int grid = (int)(want < cap ? want : cap);
+  // the launch's counters: next_slot up to fallback[0]
+  e = cudaMemsetAsync(a.next_slot, 0, (size_t)(a.fallback + 1 - a.next_slot) * sizeof(int32_t), s);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, kWarps * 32, smem, s>>>(a);
+  return launched();
 }
 
 }  // namespace

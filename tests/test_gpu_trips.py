@@ -1,0 +1,94 @@
+"""Barrier-free sweep by trip maps (csrc/trip.cuh) against the oracle, at the
+sizes where they can go wrong: trips around the shortest it takes and the 32
+iterations of a batch, bodies up to 32 records, offsets up to the farthest a
+map carries and past it, waits on outer loops' producers, more inputs than a
+map holds, and thresholds that name other increments, which the walk takes."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from tests.test_gpu_parity import ALL_MODES, compare_all
+
+pytestmark = pytest.mark.gpu
+
+PRM = dict(ii=2, c_branch=3, c_regop=2)
+
+
+@pytest.fixture(scope="module")
+def sg():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_13757_gb300 import build
+    build.build()
+    import paper_2608_13757_gb300 as m
+    return m
+
+
+def program(trips, records, engines, density, k_max, rng):
+    """Leaf loop of `records` instructions inside a loop, its waits carried at
+    offsets 0..k_max, from and to the loop around it."""
+    b = workloads.ProgramBuilder(engines)
+    eng = lambda: int(rng.integers(0, engines))
+    lat = lambda: int(rng.integers(1, 200))
+    A = b.loop(0, 0, [len(trips)])
+    a0, a1 = b.instr(A, 0, eng(), lat()), b.instr(A, 1, eng(), lat())
+    L = b.loop(A, 2, trips)
+    xs = [b.instr(L, i, eng(), lat()) for i in range(records)]
+    a2 = b.instr(A, 3, eng(), lat())
+    for i in range(records):
+        if i and rng.random() < density:
+            b.dep(xs[int(rng.integers(0, i))], xs[i], 0)
+        if rng.random() < density:
+            b.dep(xs[int(rng.integers(0, records))], xs[i], int(rng.integers(1, k_max + 1)))
+        if rng.random() < density / 3:
+            b.dep((a0, a1)[i & 1], xs[i], 0)
+    b.dep(xs[-1], a2, 0)
+    b.dep(xs[0], a0, 1)
+    b.dep(a2, xs[0], 1)
+    return b.batch()
+
+
+def batch_of(rng):
+    trips = [[40] + [t, t + 1, 0, 64, t] for t in (1, 3, 4, 31, 32, 33, 65)]
+    shapes = [(1, 1, 0.9, 1), (2, 2, 0.9, 3), (5, 3, 0.6, 4), (16, 4, 0.4, 2), (17, 5, 0.3, 3), (32, 8, 0.15, 2),
+              (32, 2, 0.8, 2), (31, 12, 0.2, 1)]
+    return workloads.concat([program(t, *s, rng) for t in trips for s in shapes])
+
+
+@pytest.mark.parametrize("seed", range(2))
+def test_trip_edges(sg, seed):
+    batch = batch_of(np.random.default_rng(seed))
+    compare_all(sg, batch, timeline=True, modes=ALL_MODES, params=oracle.sim_params(**PRM))
+
+
+def test_trip_costs(sg):
+    batch = batch_of(np.random.default_rng(5))
+    compare_all(sg, batch, timeline=True, modes=ALL_MODES,
+                params=oracle.sim_params(licm=1, cse=1, trip_register_elision=1, **PRM))
+
+
+@pytest.mark.parametrize("mode", [oracle.COUNT, oracle.PERLOOP])
+def test_waits_on_other_increments(sg, mode):
+    """Thresholds moved to earlier increments, to none and past the end."""
+    import torch
+    rng = np.random.default_rng(9)
+    batch = workloads.concat([program([40, 50, 33, 70], 16, 4, 0.4, 2, rng) for _ in range(16)])
+    h = sg.sync_load_programs(batch)
+    want = oracle.thresholds(batch, mode).copy()
+    own = np.repeat(np.arange(batch.n_deps), h.pair_counts)
+    prog = np.searchsorted(batch.prog_dep_ptr, own, side="right") - 1
+    for p in range(15):
+        at = rng.choice(np.flatnonzero((prog == p) & (want > 0)))
+        want[at] = max(0, want[at] + (-1, -9, -want[at], 10 ** 6, 1)[p % 5])
+    thr = sg.sync_eval_thresholds(h, mode)
+    thr[torch.from_numpy(h.unpadded_index()).to(thr.device)] = torch.from_numpy(want).to(thr.device)
+    ref = oracle.simulate(batch, want, mode, oracle.BARRIER_FREE)
+    r = sg.sync_simulate(h, mode, thr)
+    P = batch.n_programs
+    assert np.array_equal(r.status.cpu().numpy()[:P], ref.status)
+    assert np.array_equal(r.makespan.cpu().numpy()[:P], ref.makespan)
+    assert np.array_equal(r.checksum.cpu().numpy()[:P].view(np.uint64), ref.checksum)
+    assert (ref.status == 0).any() and (ref.status != 0).any()
+    h.close()
