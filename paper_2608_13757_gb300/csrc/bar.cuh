@@ -280,9 +280,20 @@ __device__ __forceinline__ void bar_counts(const SweepArgs& a, int p, const Prog
   if (lane == 0) a.bar.counted[p] = 1;
 }
 
-// The classes of program p's waits, from each one's first visit.  False: a
-// wait is neither on an earlier interval nor on its own producer.
+// The wait value of dependency D at the consumer's iteration g, whose
+// S-iteration is gs, computed (fused), and whether Eq. (1)'s minimum is it.
 template <int MODE>
+__device__ __forceinline__ int32_t bar_value(const SweepArgs& a, const DepInfo& D, int32_t g, int32_t gs, bool& bad) {
+  const int32_t st = D.src < 0 ? 0 : __ldg(a.bar.derived + (D.up == 0 ? D.src + g : D.tstart + gs));
+  const int32_t T = wait_value(a, D, gs, st, MODE);
+  bad = bad || (a.chk_counts && minimum(a, D, gs, st, MODE) != T);
+  return T;
+}
+
+// The classes of program p's waits, from each one's first visit.  False: a
+// wait is neither on an earlier interval nor on its own producer (or, fused,
+// differs from the checked minimum: the walk tallies it).
+template <int MODE, bool FUSED>
 __device__ bool bar_classes(const SweepArgs& a, const ProgInfo& pi, int lane) {
   const BarProg b = bar_prog(pi);
   bool bad = false;
@@ -294,7 +305,7 @@ __device__ bool bar_classes(const SweepArgs& a, const ProgInfo& pi, int lane) {
     const int32_t pe = MODE == SYNC_THR_PERENGINE ? bar_engine_pub(a, b, bd, 0) : 0;
     int32_t pub, own;
     bar_pub<MODE>(a, D, bd, gs, pe, pub, own);
-    const int32_t T = __ldg(a.thr + D.seg_off);
+    const int32_t T = FUSED ? bar_value<MODE>(a, D, 0, gs, bad) : __ldg(a.thr + D.seg_off);
     const bool in = T > pub;
     bad = bad || (in && (bd.prod_op < 0 || T != own));
     a.bar.bind[r] = in ? 1 : 0;
@@ -391,14 +402,14 @@ __device__ __forceinline__ bool bar_in_time(const SweepArgs& a, const ProgInfo& 
 }
 
 // Program p's plan by one warp; false: it has to be swept.
-template <int MODE>
+template <int MODE, bool FUSED>
 __device__ __noinline__ bool bar_plan(const SweepArgs& a, int p, int32_t* at, int lane) {
   const ProgInfo pi = a.prog[p];
   const BarProg b = bar_prog(pi);
   bool ok = pi.n_inst >= a.bar.min_inst && bar_in_time<MODE>(a, pi);
   if (ok) {
     bar_counts(a, p, pi, lane);
-    ok = bar_classes<MODE>(a, pi, lane);
+    ok = bar_classes<MODE, FUSED>(a, pi, lane);
   }
   __syncwarp();
   for (int l = pi.loop_base + pi.nloops - 1; ok && l >= pi.loop_base; --l)
@@ -416,7 +427,7 @@ __device__ __noinline__ bool bar_plan(const SweepArgs& a, int p, int32_t* at, in
 // iterations per lane, which one broadcast of a record serves.  `at`: 32
 // ints of shared memory.  Returns whether a wait is outside its class
 // (warp-uniform).
-template <int MODE>
+template <int MODE, bool FUSED>
 __device__ __forceinline__ bool bar_waits(const SweepArgs& a, const BarProg& b, int32_t g0, int32_t g1,
                                           const int4 op, int32_t* at, int lane) {
   // the chunk's dependencies, one per lane
@@ -448,7 +459,7 @@ __device__ __forceinline__ bool bar_waits(const SweepArgs& a, const BarProg& b, 
       mul = MODE == SYNC_THR_PERLOOP ? D.N : 1;
       add = in ? (MODE == SYNC_THR_PERLOOP ? D.K : 1) : MODE == SYNC_THR_PERLOOP ? bd.b[1] : bd.b[0];
       if (bd.prod_fixed) add += in ? 0 : mul * bd.delta;
-      for (int32_t g = g0; g < g1; g += 32)   // the thresholds' lines, while the others' records load
+      for (int32_t g = g0; !FUSED && g < g1; g += 32)   // the thresholds' lines, while the others' records load
         asm volatile("prefetch.global.L2 [%0];" ::"l"(a.thr + seg + g));
       kind = (!(bd.prod_fixed) ? 3 : bd.cons_fixed ? 0 : D.src < 0 ? 2 : 1) | (in ? 4 : 0);
     }
@@ -456,7 +467,7 @@ __device__ __forceinline__ bool bar_waits(const SweepArgs& a, const BarProg& b, 
     for (int k = 0; k < n; ++k) {
       const int kk = __shfl_sync(kBarFull, kind, k);
       const int64_t so = __shfl_sync(kBarFull, seg, k);
-      if (MODE == SYNC_THR_PERENGINE || (kk & 3) == 3) {
+      if (FUSED || MODE == SYNC_THR_PERENGINE || (kk & 3) == 3) {
         const int rr = __shfl_sync(kBarFull, r, k);
         const DepInfo D = a.bar.dep[__ldg(a.bar.ddep + rr)];
         const BarDep bd = a.bar.bdep[rr];
@@ -465,7 +476,7 @@ __device__ __forceinline__ bool bar_waits(const SweepArgs& a, const BarProg& b, 
           const int32_t pe = MODE == SYNC_THR_PERENGINE ? bar_engine_pub(a, b, bd, g) : 0;
           int32_t pub, own;
           bar_pub<MODE>(a, D, bd, gs, pe, pub, own);
-          const int32_t T = __ldg(a.thr + so + g);
+          const int32_t T = FUSED ? bar_value<MODE>(a, D, g, gs, bad) : __ldg(a.thr + so + g);
           bad = bad || (kk & 4 ? T != own : T > pub);
         }
         continue;
@@ -658,7 +669,7 @@ __device__ __noinline__ unsigned long long bar_times_any(const SweepArgs& a, con
   return chk;
 }
 
-template <int MODE, bool TL>
+template <int MODE, bool TL, bool FUSED>
 __device__ __forceinline__ bool bar_body(const SweepArgs& a, int tile, int l, const BarLoop& B, int32_t* at, int lane,
                                          unsigned long long& chk) {
   const ProgInfo& pi = a.prog[B.prog];
@@ -671,7 +682,7 @@ __device__ __forceinline__ bool bar_body(const SweepArgs& a, int tile, int l, co
   bool bad = false;
   for (int32_t c = r0; c < r1; c += 32) {
     if (c > r0) op = c + lane < r1 ? __ldg(a.bar.ops + c + lane) : make_int4(OP_END, 0, 0, 0);
-    if (__ballot_sync(kBarFull, op.x >= 0 && op.z > 0)) bad = bar_waits<MODE>(a, b, g0, g1, op, at, lane) || bad;
+    if (__ballot_sync(kBarFull, op.x >= 0 && op.z > 0)) bad = bar_waits<MODE, FUSED>(a, b, g0, g1, op, at, lane) || bad;
   }
   const int h = B.host;
   const BarLoop BH = a.bar.bl[h];
@@ -697,13 +708,13 @@ __device__ __forceinline__ void bar_add(const SweepArgs& a, int p, unsigned long
 
 // One tile in the sweep's launch.  Returns the program when this was its
 // last tile and a wait differed (it has to be swept), else -1.
-template <int MODE, bool TL>
+template <int MODE, bool TL, bool FUSED>
 __device__ __forceinline__ int bar_tile(const SweepArgs& a, int tile, int32_t* at, int lane) {
   const int l = __ldg(a.bar.tile_loop + tile);
   const BarLoop B = a.bar.bl[l];
   if (__ldcg(a.bar.left + B.prog) < 0) return -1;
   unsigned long long chk = 0;
-  const bool bad = bar_body<MODE, TL>(a, tile, l, B, at, lane, chk);
+  const bool bad = bar_body<MODE, TL, FUSED>(a, tile, l, B, at, lane, chk);
   bar_add(a, B.prog, chk, lane);
   __threadfence();                 // the tile's results before its count, for a sweep of the program
   __syncwarp();

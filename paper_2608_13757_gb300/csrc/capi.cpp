@@ -1147,9 +1147,9 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
   w.maps = maps;
   if (variant != SYNC_SIM_BARRIER && (maps || h->n_split > 0)) w.bar = h->bar;   // trip maps read the dependencies' tables
   const bool barrier = variant == SYNC_SIM_BARRIER;
-  // barrier scheme (array thresholds): by intervals, in the sweep's launch or,
-  // with split programs, in launches of its own
-  if (!fused && barrier && h->bar.on && h->max_inst >= kBarMinInst) {
+  // barrier scheme: by intervals, in the sweep's launch or, with split
+  // programs, in launches of its own
+  if (barrier && h->bar.on && h->max_inst >= kBarMinInst) {
     w.bar = h->bar;
     if (const int r = sweep_ring_for(a.sem_cap, a.frame_depth, false, kBarRingBytes)) w.ring = r;
     w.bar.min_inst = kBarMinInst;

@@ -11,8 +11,11 @@ cudaError_t launch3(const SweepArgs& a, size_t smem, int num_sms, cudaStream_t s
   auto run = [&](auto kern) { return run_sweep(kern, a, items, smem, num_sms, s); };
   if constexpr (BB) {
     if (a.bar.on && a.bar.n_tiles > items) items = a.bar.n_tiles;
-    if (a.bar.on || a.bar.todo)
+    if (a.bar.on || a.bar.todo) {
+      if (a.dep)
+        return a.issue ? run(k_sweep<MODE, true, true, true, false, true>) : run(k_sweep<MODE, true, false, true, false, true>);
       return a.issue ? run(k_sweep<MODE, true, true, false, false, true>) : run(k_sweep<MODE, true, false, false, false, true>);
+    }
   }
   if (a.dep) return a.issue ? run(k_sweep<MODE, BB, true, true>) : run(k_sweep<MODE, BB, false, true>);
   return a.issue ? run(k_sweep<MODE, BB, true, false>) : run(k_sweep<MODE, BB, false, false>);

@@ -53,7 +53,7 @@ struct Frame { int32_t loop, item, g, g_end; };
 
 // A leaf loop's trip map in shared memory, per warp (trip.cuh).
 constexpr int kTripCols = 24;               // inputs
-constexpr int kTripInts = 2 * 32 * kTripCols + 32 * (kTripCols + 1) + 64 + 4 * 32 + 8 * 32 + 16;
+constexpr int kTripInts = 2 * 32 * kTripCols + 32 * (kTripCols + 1) + 64 + 4 * 32 + 8 * 32 + 32 + 16;
 
 // Shared memory of one warp (program), 16-byte aligned.
 __host__ __device__ __forceinline__ size_t warp_bytes(int sem_cap, int frame_depth, int ring, bool maps) {
@@ -846,8 +846,8 @@ __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, c
                                         const int4 one, int32_t lo, int32_t hi, int32_t ctag, int lane, int lc,
                                         int32_t iter_cost, unsigned long long& chk) {
   if (hi - lo == 1 && one.y == 1) return run_single<MODE, BB, TL, FUSED>(a, S, pi, one, lo, lane, lc, chk);
-  if (MAPS && !FUSED) {
-    lo = run_trip<MODE, TL>(a, S, pi, one, lo, hi, lane, iter_cost, chk);
+  if (MAPS) {
+    lo = run_trip<MODE, TL, FUSED>(a, S, pi, one, lo, hi, lane, lc, iter_cost, chk);
     if (lo == hi) return 0;
   }
   const int32_t copies = ch.z;
@@ -887,9 +887,9 @@ __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, c
 // PieceArgs) instead of whole programs: item = piece * probes + probe; the
 // walk starts inside the body of the piece's loop L at its first iteration
 // start and ends after its last iteration.
-// BAR (barrier scheme, array thresholds): programs by intervals (bar.cuh),
-// and by the walk only those the intervals leave.  MAPS (barrier-free): leaf
-// trips by their maps (trip.cuh).
+// BAR (barrier scheme): programs by intervals (bar.cuh), and by the walk only
+// those the intervals leave.  MAPS (barrier-free): leaf trips by their maps
+// (trip.cuh).
 template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false, bool BAR = false, bool MAPS = false>
 __global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_sweep(const __grid_constant__ SweepArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -949,7 +949,7 @@ __global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_
       }
       if (BAR && a.bar.on) {
         const int q = __ldg(a.order + slot);
-        const bool ok = bar_plan<MODE>(a, q, S.nn, lane);
+        const bool ok = bar_plan<MODE, FUSED>(a, q, S.nn, lane);
         __threadfence();
         __syncwarp();
         if (lane == 0) atomicAdd(a.bar.plans, 1);
@@ -958,7 +958,7 @@ __global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_
       }
     } else {
       if (tile >= a.bar.n_tiles) break;
-      if (planned) left = bar_tile<MODE, TL>(a, tile, S.nn, lane);
+      if (planned) left = bar_tile<MODE, TL, FUSED>(a, tile, S.nn, lane);
       else if (lane == 0) a.status[a.bar.bl[a.bar.tile_loop[tile]].prog] = SYNC_PROG_ROUND_GUARD;
       tile += gridDim.x * kWarps;
       if (left < 0) continue;

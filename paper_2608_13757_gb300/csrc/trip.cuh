@@ -35,7 +35,8 @@ constexpr int kTripCol = kTripDep + 32;             // [32] kind | lane << 4 | d
 constexpr int kTripRec = kTripCol + 32;             // [32] engine | records of it << 8 | rank among them << 16
 constexpr int kTripInc = kTripRec + 32;             // [32] semaphore | rank << 16 | increments << 24, or -1
 constexpr int kTripOut = kTripInc + 32;             // [32] int4 x 2: a record's outputs in this trip (see trip_times)
-constexpr int kTripHead = kTripOut + 8 * 32;        // {chunk, inputs (0: none yet), dependencies, iterations
+constexpr int kTripR = kTripOut + 8 * 32;           // [32] a dependency's consumer-grouped index (fused)
+constexpr int kTripHead = kTripR + 32;             // {chunk, inputs (0: none yet), dependencies, iterations
                                                     //  walked (< 0: never), maps allowed}
 static_assert(kTripHead + 16 == kTripInts, "trip map layout");
 enum : int { TD_CHUNK = 0, TD_CARRIED = 1, TD_OUTER = 2 };                       // dependencies
@@ -94,6 +95,7 @@ __device__ __noinline__ bool trip_build(const SweepArgs& a, int32_t* map, const 
       }
     }
     reinterpret_cast<int64_t*>(map + kTripSeg)[pre + j] = __ldg(a.dseg + r);
+    map[kTripR + pre + j] = r;
     map[kTripDep + pre + j] = kind | k << 2 | rank << 4 | inc << 10 | s << 16;
     map[kTripCol + pre + j] = lane | p << 8;       // until the columns are known
   }
@@ -249,9 +251,11 @@ __device__ __forceinline__ void trip_times(const SweepArgs& a, const WarpSmem& S
 // Iterations lo .. hi-1 of a trip by the map of its body's chunk `ch`; the
 // first iteration start has been charged.  Returns the first iteration it
 // did not take (the state is then as that iteration starts).
-template <int MODE, bool TL>
+// FUSED: the thresholds are computed (walk level lc), and compared with the
+// Eq. (1) minimum if asked; a trip where they differ is walked, which tallies.
+template <int MODE, bool TL, bool FUSED>
 __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& S, const ProgInfo& pi, const int4 ch,
-                                            int32_t lo, int32_t hi, int lane, int32_t iter_cost,
+                                            int32_t lo, int32_t hi, int lane, int lc, int32_t iter_cost,
                                             unsigned long long& chk) {
   int32_t* map = S.map;
   const int32_t total = hi - lo;
@@ -288,8 +292,15 @@ __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& 
     const int32_t pub = S.semv[D >> 16];
     dk = (D >> 2) & 3;
     if ((D & 3) == TD_OUTER) {
-      T0 = __ldg(a.thr + seg);
-      bad = T0 > pub;
+      if (FUSED) {
+        const DepInfo F = a.dep[__ldg(a.ddep + map[kTripR + lane])];
+        const int2 v = S.lvl[lc - F.up];
+        T0 = wait_value(a, F, v.x, v.y, MODE);
+        bad = a.chk_counts && minimum(a, F, v.x, v.y, MODE) != T0;
+      } else {
+        T0 = __ldg(a.thr + seg);
+      }
+      bad = bad || T0 > pub;
     } else {
       step = (D >> 10) & 63;
       T0 = pub + ((D >> 4) & 63) - dk * step;
@@ -325,11 +336,23 @@ __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& 
     out[1] = make_int4(S.nn[rec & 255] + (rec >> 16), (rec >> 8) & 255, rec & 255, __ldg(a.lrec + ch.x + lane).x);
   }
   __syncwarp();
+  if (FUSED) {                              // all iterations first: the walk cannot take over in a trip
+    for (int d = 0; d < nd; ++d) {
+      const DepInfo F = a.dep[__ldg(a.ddep + map[kTripR + d])];
+      if (F.up > 0) continue;                // constant over the trip
+      const int32_t w0 = __shfl_sync(kFull, T0, d), st = __shfl_sync(kFull, step, d);
+      for (int32_t j = lane; j < total; j += 32) {
+        const int32_t T = wait_value(a, F, lo + j, lo, MODE);
+        bad = bad || T != (j < F.k ? 0 : w0 + j * st) || (a.chk_counts && minimum(a, F, lo + j, lo, MODE) != T);
+      }
+    }
+    if (__ballot_sync(kFull, bad)) return lo;
+  }
   const int groups = (nc + 3) >> 2;
   int32_t done = 0;
   for (; done < total; done += 32) {
     const int32_t nb = min(32, total - done), j = done + lane;
-    for (int d = 0; d < nd; d += 4) {
+    for (int d = 0; !FUSED && d < nd; d += 4) {
       int32_t T[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
