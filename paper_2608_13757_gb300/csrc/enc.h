@@ -70,8 +70,7 @@ struct alignas(16) ProgInfo {
   int64_t el_stmt;    // of these, those of loops that carry no offset > 0 (whose trip
   int64_t el_iter;    // register can be elided)
   int64_t pair_levels;  // sum over pairs of the per-engine wait's extra levels
-  int64_t fb_iters;   // iterations ended by a barrier-fallback barrier (barrier-free);
-                      // > 0: simulated by the per-engine kernel
+  int64_t fb_iters;   // iterations ended by a barrier-fallback barrier (barrier-free)
   int64_t licm_upd;   // LICM (per-engine waits): cached-sum updates, summed over the
                       // (loop, engine) rows of their counts times the loop's iterations
   int64_t lv_pairs;   // pairs of per-engine waits whose producer loop has depth > 1
@@ -91,6 +90,8 @@ struct alignas(16) ProgInfo {
 // into straight-line segments; items [plan_ptr[l], plan_ptr[l+1]):
 //   {ITEM_SEG, first chunk, chunks, w}
 //   {ITEM_LOOP, child loop (global id), child's elidable-trip-register flag, 0}
+//   {ITEM_BARRIER, 0, 0, 0}: last in a body whose iterations end with a
+//     barrier-fallback barrier (barrier-free)
 // with w >= 0 a multi-iteration chunk, w <= -2 (the body's last segment) a
 // chunk of that segment and the next iteration's first (chunk -2 - w), -1
 // neither.  A chunk holds up to 32 datapath records of one segment (all
@@ -107,7 +108,7 @@ struct alignas(16) ProgInfo {
 //     flags bit 0: first record of its engine in a copy >= 1 (an iteration
 //     start precedes it); bit 1: last lane of its engine's run
 //   lsem per mode {semaphore, stride, koff, levels} as the simulator's records.
-enum : int32_t { ITEM_SEG = 0, ITEM_LOOP = 1 };
+enum : int32_t { ITEM_SEG = 0, ITEM_LOOP = 1, ITEM_BARRIER = 2 };
 constexpr int32_t LANE_ITER_START = 1;
 constexpr int32_t LANE_RUN_LAST = 2;
 

@@ -1033,9 +1033,11 @@ struct ProgBuilder {
           add_item(make_int4(ITEM_LOOP, l0 + m, FILL ? O.lflag[l0 + m] : 0, 0));
         }
       }
+      // a fallback barrier ends the iteration: not a leaf for the sweep's loops
+      if (S.fbar[l0 + l]) add_item(make_int4(ITEM_BARRIER, 0, 0, 0));
       // a short body with no child loop: a template of several iterations
       const int32_t L = bp[l + 1] - bp[l];
-      if (nloops == 0 && nseg == 1 && L >= 1 && L <= 16) {
+      if (nloops == 0 && nseg == 1 && L >= 1 && L <= 16 && !S.fbar[l0 + l]) {
         const int32_t k = 32 / L;
         if constexpr (!FILL) {                    // COUNT: every record in each of k copies
           c[BC_LANES] += (int64_t)k * L;
@@ -1067,7 +1069,7 @@ struct ProgBuilder {
       int32_t lb = b1;
       while (bd[lb - 1] >= 0) --lb;                   // just past the last one
       const int32_t na = fa - b0, nb = b1 - lb;
-      if (na < 1 || nb < 1 || na + nb > 32) continue;
+      if (na < 1 || nb < 1 || na + nb > 32 || S.fbar[l0 + l]) continue;
       if constexpr (!FILL) {
         c[BC_LANES] += na + nb;
         c[BC_CHUNKS]++;
@@ -1102,7 +1104,7 @@ struct ProgBuilder {
       for (int64_t i = plan_first; i < c[BC_PLAN]; ++i) {
         const int4 v = O.plan[i];
         if (v.x != ITEM_LOOP) {                   // a segment: its first chunk's record
-          O.paux[i] = O.chunks[v.y];
+          O.paux[i] = v.x == ITEM_SEG ? O.chunks[v.y] : make_int4(0, 0, 0, 0);
           continue;
         }
         const int32_t m = v.y - l0;
@@ -1112,6 +1114,8 @@ struct ProgBuilder {
         if (e - b == 1 && O.plan[b].x == ITEM_SEG) {
           if (O.plan[b].z == 1) bf = bb = O.plan[b].y;
           if (O.plan[b].w >= 0) bf = O.plan[b].w;
+        } else if (e - b == 2 && O.plan[b].x == ITEM_SEG && O.plan[b].z == 1 && O.plan[b + 1].x == ITEM_BARRIER) {
+          bb = O.plan[b].y;                       // the barrier scheme has that barrier already
         }
         const int64_t rp = S.srp[sr(m, 0)];
         O.paux[i] = make_int4((int32_t)(uint32_t)(rp & 0xffffffffu), (int32_t)(rp >> 32), bf, bb);

@@ -2,9 +2,8 @@
 //
 // Under a common loop tree every engine meets the same loop statements and
 // iteration boundaries, so one walker per program can visit the tree once for
-// all engines (programs whose engines run their own trip counts, and
-// barrier-free the programs with the barriers of the non-allocatable
-// fallback, go straight to the per-engine kernel).  The body of each loop is cut at its child loops into
+// all engines (programs whose engines run their own trip counts go straight
+// to the per-engine kernel).  The body of each loop is cut at its child loops into
 // straight-line segments; a segment is taken as one chunk of up to 32 datapath
 // records (more chunks if longer), or -- barrier-free, for a short innermost
 // body -- as several consecutive iterations at once.  The chunk's lanes are
@@ -1000,10 +999,9 @@ __global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_
     };
     BbRep no_rep;                     // a segment's chunk is neither replayed
     BfPred no_pred;                   // nor predicted
-    // engines on their own trips (no common walk), or barrier-free with the
-    // barriers of the non-allocatable fallback: the per-engine kernel (split
-    // programs have neither; their time bound was checked by the validation)
-    if (!PIECE && (pi.divergent || (!BB && pi.fb_iters > 0))) {
+    // engines on their own trips (no common walk): the per-engine kernel
+    // (split programs have none; their time bound was checked by the validation)
+    if (!PIECE && pi.divergent) {
       if (lane == 0) {
         a.status[p] = SIM_FALLBACK;
         a.fallback[1 + atomicAdd(a.fallback, 1)] = p;
@@ -1129,6 +1127,11 @@ __global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_
           pend = ce;
         }
         __syncwarp();
+        continue;
+      }
+      if (it.x == ITEM_BARRIER) {                      // a fallback barrier ends the iteration
+        if (!BB) barrier_all(S, pi.ne, a.prm.c_barrier, lane);
+        ++item;
         continue;
       }
       // a straight-line segment
