@@ -307,7 +307,7 @@ __device__ bool bar_classes(const SweepArgs& a, const ProgInfo& pi, int lane) {
     bar_pub<MODE>(a, D, bd, gs, pe, pub, own);
     const int32_t T = FUSED ? bar_value<MODE>(a, D, 0, gs, bad) : __ldg(a.thr + D.seg_off);
     const bool in = T > pub;
-    bad = bad || (in && (bd.prod_op < 0 || T != own));
+    bad = bad || (in && (!bd.in_seg || T != own));
     a.bar.bind[r] = in ? 1 : 0;
   }
   return !__ballot_sync(kBarFull, bad);

@@ -840,7 +840,7 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
     code_unrolled += s.code_unrolled;
     n_bar_deps += s.n_bar_deps;
     h.max_inst = std::max(h.max_inst, s.n_inst);
-    h.n_stmt += s.n_stmt;
+    for (int k = 0; k < 2; ++k) h.n_stmt[k] += s.n_stmt[k];
     ne_max = std::max(ne_max, s.ne);
     depth_max = std::max(depth_max, s.depth_max);
     ord_overflow |= s.ord_overflow;
@@ -1145,6 +1145,7 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
   w.dep = a.dep; w.ddep = a.ddep; w.path = a.path; w.ord = a.ord;
   w.chk_counts = a.chk_counts; w.chk_first = a.chk_first;
   w.maps = maps;
+  w.opsem = a.opsem;
   if (variant != SYNC_SIM_BARRIER && (maps || h->n_split > 0)) w.bar = h->bar;   // trip maps read the dependencies' tables
   const bool barrier = variant == SYNC_SIM_BARRIER;
   // barrier scheme: by intervals, in the sweep's launch or, with split

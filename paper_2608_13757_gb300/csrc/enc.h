@@ -308,7 +308,7 @@ struct alignas(16) BarLoop {   // per loop, and a last entry (tile0: all tiles)
 //   count X + b[0]; per loop N*X + b[1]; per engine the engine's instances
 //   before C's iteration and its children so far + b2.
 struct alignas(16) BarDep {
-  int32_t prod_op;   // op record of a producer in the consumer's own segment, else -1
+  int32_t prod_op;   // producer's op record
   int32_t b[2];
   int32_t b2;
   int32_t cons_loop; // C
@@ -317,7 +317,7 @@ struct alignas(16) BarDep {
   uint8_t delta;
   uint8_t cons_fixed;  // S's iteration is C's (only fixed loops between)
   uint8_t prod_fixed;  // X = gs + delta (likewise)
-  int32_t pad_;
+  int32_t in_seg;    // the producer is in the consumer's own segment
 };
 struct BarArgs {
   int32_t on;                // 1: the sweep launch runs the intervals first (bar.cuh)
@@ -447,7 +447,8 @@ struct SweepArgs {
   CostTables cost;
   PieceArgs pcs;             // piece-parallel simulation (prog_split NULL: none)
   BarArgs bar;               // barrier scheme by intervals
-  int32_t maps;              // barrier-free: leaf trips by their maps (trip.cuh)
+  int32_t maps;              // barrier-free: trips by their maps (trip.cuh)
+  const int4* opsem;         // per-mode records, parallel to bar.ops
 };
 
 // Launchers (return the launch error, if any).
@@ -479,15 +480,18 @@ cudaError_t launch_simulate(const SimArgs& a, bool barrier, int num_sms, cudaStr
 cudaError_t launch_sweep(const SweepArgs& a, bool barrier, int num_sms, cudaStream_t s);
 size_t sweep_smem_bytes(int sem_cap, int frame_depth, int ring, bool maps);
 cudaError_t launch_sweep_maps(const SweepArgs& a, int num_sms, cudaStream_t s);
-// Whether the barrier-free sweep of a batch takes its leaf loops' trips by
-// their maps (trip.cuh; 16 warps per SM instead of 24): where the longest
-// programs bound it, and where trips hold most of the work.  Chain programs
-// (264 instances per loop statement), walked / by maps: 4864 12.7 / 8.0 ms,
-// 8192 12.9 / 9.5, 16384 14.5 / 14.6, 32768 16.4 / 21.3; depth2 (540)
-// 16384 6.9 / 4.5, attention (393) 500 94 / 29; branching trees (7) 6000
-// 0.86 / 1.24, conditionals around one instruction (1) 2432 17.0 / 20.2.
-inline bool sweep_maps(int32_t n_programs, int64_t n_instances, int64_t n_statements, int num_sms) {
-  return n_instances >= 32 * n_statements && (n_programs <= 80 * num_sms || n_instances >= 320 * n_statements);
+// Whether the barrier-free sweep of a batch takes its loops' trips by their
+// maps (trip.cuh; 16 warps per SM instead of 24): where the longest programs
+// bound it, where trips hold most of the work, and where most statements are
+// of fixed loops, which a map takes with their host's iterations.  Instances
+// per statement (not fixed), programs, walked / by maps: chain 264, 4864
+// programs 12.7 / 8.0 ms, 8192 12.9 / 9.5, 16384 14.5 / 14.6, 32768 16.4 /
+// 21.3; depth2 540, 16384 6.9 / 4.5; attention 393, 500 94 / 29; branching
+// trees 20, 6000 0.86 / 1.38; conditionals around one instruction (24 fixed
+// statements to a moving one) 65536 34.0 / 12.5.
+inline bool sweep_maps(int32_t n_programs, int64_t n_instances, const int64_t (&n_stmt)[2], int num_sms) {
+  return n_stmt[1] >= 4 * n_stmt[0] ||
+         (n_instances >= 32 * n_stmt[0] && (n_programs <= 80 * num_sms || n_instances >= 320 * n_stmt[0]));
 }
 // Piece-parallel simulation of the split programs (a.pcs), barrier-free:
 // validation, the probe runs or speculation, the composition of the pieces, and the pass that forms the instances' true times (checksums,

@@ -86,7 +86,7 @@ struct sync_programs {
   int32_t* next_slot = nullptr;     // scratch: simulator's program-slot counter
   int32_t* fallback = nullptr;      // scratch: programs handed to the per-engine kernel
   int64_t max_inst = 0;             // instances of the largest program
-  int64_t n_stmt = 0;               // loop statements one engine reaches, all programs
+  int64_t n_stmt[2] = {0, 0};       // loop statements of all programs, of moving loops and fixed ones
   syncgb::BarArgs bar{};            // barrier scheme by intervals (bar.cuh)
   int32_t* todo = nullptr;          // scratch: programs the intervals leave to the sweep
   // program-order sweep

@@ -106,6 +106,7 @@ extern "C" sync_status sync_simulate_noalloc(const sync_programs* h, sync_thr_mo
   w.sem_cap = sem_cap; w.frame_depth = frame_depth; w.ring = ring; w.lflag = h->lflag; w.paux = h->paux;
   w.cost = h->cost;
   w.maps = maps;
+  w.opsem = h->opsem + (size_t)mode * h->n_ops;
   if (maps) w.bar = h->bar;                // trip maps read the dependencies' tables
   st = cuda_error(launch_sweep(w, barrier, h->num_sms, s), "sweep simulator kernel");
   if (st != SYNC_OK) return st;

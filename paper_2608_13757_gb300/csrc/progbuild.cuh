@@ -148,7 +148,8 @@ struct BuildOut {
 // What COUNT reports per program besides the counts.
 struct alignas(16) ProgSummary {
   int64_t work;            // simulated work (the simulators' program order)
-  int64_t n_inst, n_stmt;
+  int64_t n_inst;
+  int64_t n_stmt[2];       // loop statements (on engine 0), of loops that are not fixed and of those that are
   int64_t code_looped, code_unrolled;   // static instructions (code-size proxy)
   int64_t n_bar_deps;      // barrier-fallback dependencies
   int64_t struct_bytes;    // path entries and rowptr spaces the threshold kernels read
@@ -845,7 +846,7 @@ struct ProgBuilder {
       const int32_t pc = S.prevc[x0 + cx];        // the child loop before the consumer's segment
       auto before = [&](int32_t m) { return m < 0 ? 0 : S.before[row0 + (int64_t)m * ne + ep]; };
       BarDep b{};
-      b.prod_op = -1;
+      b.prod_op = S.op_of[x0 + px];
       b.prod_fixed = S.dep_fix[d0 + k] & 1;
       b.cons_fixed = S.dep_fix[d0 + k] >> 1;
       b.ep = (uint8_t)ep;
@@ -855,7 +856,7 @@ struct ProgBuilder {
       if (ca < 0) {
         b.b[1] = before(cb < 0 ? pc : cb);
         b.b[0] = S.rank[x0 + px] <= b.b[1] ? 1 : 0;
-        if (cb < 0 && S.prevc[x0 + px] == pc) b.prod_op = S.op_of[x0 + px];
+        b.in_seg = cb < 0 && S.prevc[x0 + px] == pc;
       } else if (cb < 0) {
         b.delta = pc >= 0 && S.cidx[l0 + ca] <= S.cidx[l0 + pc] ? 1 : 0;
       } else {
@@ -1165,7 +1166,7 @@ struct ProgBuilder {
       for (int i = 0; i < kBuildCounts; ++i) A.count[(int64_t)p * kBuildCounts + i] = ok ? c[i] : 0;
       sm.ne = ne;
       sm.n_inst = pi.n_inst;
-      sm.n_stmt = pi.n_stmt;
+      for (int32_t l = 1; l < nl; ++l) sm.n_stmt[fixed(l)] += tot(par[l], 0);
       sm.work = pi.n_inst + pi.n_pairs + (pi.n_stmt + pi.n_iter) * pi.ne;
       sm.splittable = !d.div && pi.fb_iters == 0;
       A.sum[p] = sm;

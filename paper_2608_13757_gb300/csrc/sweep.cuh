@@ -50,9 +50,9 @@ constexpr int SIM_FALLBACK = 9;             // internal: handed to the per-engin
 
 struct Frame { int32_t loop, item, g, g_end; };
 
-// A leaf loop's trip map in shared memory, per warp (trip.cuh).
+// A loop's trip map in shared memory, per warp (trip.cuh).
 constexpr int kTripCols = 24;               // inputs
-constexpr int kTripInts = 2 * 32 * kTripCols + 32 * (kTripCols + 1) + 64 + 4 * 32 + 8 * 32 + 32 + 16;
+constexpr int kTripInts = 2 * 32 * kTripCols + 32 * (kTripCols + 1) + 64 + 7 * 32 + 8 * 32 + 16;
 
 // Shared memory of one warp (program), 16-byte aligned.
 __host__ __device__ __forceinline__ size_t warp_bytes(int sem_cap, int frame_depth, int ring, bool maps) {
@@ -840,15 +840,11 @@ namespace {
 // in registers; the next chunk's thresholds load while this one runs.
 // `one`: the chunk holding one iteration's whole body; with a single
 // iteration of one record it is applied directly.
-template <int MODE, bool BB, bool TL, bool FUSED, bool MAPS>
+template <int MODE, bool BB, bool TL, bool FUSED>
 __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, const ProgInfo& pi, const int4 ch,
                                         const int4 one, int32_t lo, int32_t hi, int32_t ctag, int lane, int lc,
                                         int32_t iter_cost, unsigned long long& chk) {
   if (hi - lo == 1 && one.y == 1) return run_single<MODE, BB, TL, FUSED>(a, S, pi, one, lo, lane, lc, chk);
-  if (MAPS) {
-    lo = run_trip<MODE, TL, FUSED>(a, S, pi, one, lo, hi, lane, lc, iter_cost, chk);
-    if (lo == hi) return 0;
-  }
   const int32_t copies = ch.z;
   const bool have = lane < ch.y;
   LaneRec L;
@@ -887,7 +883,7 @@ __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, c
 // walk starts inside the body of the piece's loop L at its first iteration
 // start and ends after its last iteration.
 // BAR (barrier scheme): programs by intervals (bar.cuh), and by the walk only
-// those the intervals leave.  MAPS (barrier-free): leaf trips by their maps
+// those the intervals leave.  MAPS (barrier-free): trips by their maps
 // (trip.cuh).
 template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false, bool BAR = false, bool MAPS = false>
 __global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_sweep(const __grid_constant__ SweepArgs a) {
@@ -1109,19 +1105,21 @@ __global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_
           __syncwarp();
           if (lane < pi.ne) S.t[lane] += child_ic;    // the first iteration starts
           __syncwarp();
+          // iterations by the loop's trip map; the others
+          const int32_t from = MAPS ? run_trip<MODE, TL, FUSED>(a, S, pi, it.y, lo, hi, lane, sp + 1, child_ic, chk) : lo;
+          if (MAPS && from == hi) continue;
           if (body_chunk >= 0) {
             // one iteration of one record: applied directly; otherwise a
             // loop around one chunk: all its iterations in registers
-            verdict = run_loop<MODE, BB, TL, FUSED, MAPS>(a, S, pi, chb, one, lo,
-                                                    hi, ++ctag, lane, sp + 1, child_ic, chk);
+            verdict = run_loop<MODE, BB, TL, FUSED>(a, S, pi, chb, one, from, hi, ++ctag, lane, sp + 1, child_ic, chk);
             if (verdict) break;
             continue;
           }
           const int32_t cb = __ldg(a.plan_ptr + it.y), ce = __ldg(a.plan_ptr + it.y + 1);
           if (lane == 0) S.frames[sp] = Frame{loop, item, g, g_end};
           ++sp;
-          if (FUSED && lane == 0) S.lvl[sp] = make_int2(lo, lo);
-          loop = it.y; item = 0; g = lo; g_end = hi;
+          if (FUSED && lane == 0) S.lvl[sp] = make_int2(from, lo);
+          loop = it.y; item = 0; g = from; g_end = hi;
           iter_cost = child_ic;
           pbeg = cb;
           pend = ce;

@@ -1,6 +1,10 @@
-// Barrier-free sweep: the iterations of a leaf loop's trip by its max-plus map.
+// Barrier-free sweep: the iterations of a loop's trip by its max-plus map,
+// for loops whose iterations are one straight line of at most 32 records: no
+// child loops but fixed ones (which run exactly once on every visit, so
+// their records' instances are the loop's iterations and they cost every
+// engine the same each time).
 //
-// With its in-chunk waits fixed, every issue and retire of an iteration is a
+// With its waits inside an iteration fixed, every issue and retire of an iteration is a
 // maximum, over the engines' cursors and last retires at its start and the
 // times its waits on earlier increments are satisfied (the map's inputs), of
 // that value plus a sum of costs along a path (all costs >= 0, no constant
@@ -30,32 +34,84 @@ constexpr int kTripRow = kTripCols + 1;     // odd: a lane per row without bank 
 // the warp's ints (kTripInts)
 constexpr int kTripIn = 2 * 32 * kTripCols;         // [32][kTripRow] inputs per iteration
 constexpr int kTripSeg = kTripIn + 32 * kTripRow;   // [32] int64: a dependency's thresholds
-constexpr int kTripDep = kTripSeg + 64;             // [32] kind | k << 2 | rank << 4 | increments << 10 | semaphore << 16
+constexpr int kTripDep = kTripSeg + 64;             // [32] kind | k << 2 | rank << 4 | increments << 10 | semaphore << 16 | S in the body << 31
 constexpr int kTripCol = kTripDep + 32;             // [32] kind | lane << 4 | dependency << 12 | k << 20 | engine << 24
 constexpr int kTripRec = kTripCol + 32;             // [32] engine | records of it << 8 | rank among them << 16
 constexpr int kTripInc = kTripRec + 32;             // [32] semaphore | rank << 16 | increments << 24, or -1
 constexpr int kTripOut = kTripInc + 32;             // [32] int4 x 2: a record's outputs in this trip (see trip_times)
-constexpr int kTripR = kTripOut + 8 * 32;           // [32] a dependency's consumer-grouped index (fused)
-constexpr int kTripHead = kTripR + 32;             // {chunk, inputs (0: none yet), dependencies, iterations
-                                                    //  walked (< 0: never), maps allowed}
+constexpr int kTripR = kTripOut + 8 * 32;           // [32] a dependency's consumer-grouped index
+constexpr int kTripX = kTripR + 32;                 // [32] a record's global instruction
+constexpr int kTripTail = kTripX + 32;              // [32] an engine's control costs after its last record (all, without one)
+constexpr int kTripHead = kTripTail + 32;           // {loop, inputs (0: none yet), dependencies | records << 8,
+                                                    //  iterations walked (< 0: never), maps allowed}
 static_assert(kTripHead + 16 == kTripInts, "trip map layout");
 enum : int { TD_CHUNK = 0, TD_CARRIED = 1, TD_OUTER = 2 };                       // dependencies
 enum : int { TC_CURSOR = 0, TC_RETIRE = 1, TC_CARRIED = 2, TC_OUTER = 3, TC_NONE = 4 };   // inputs
 
-// Builds the map of chunk ch (one iteration of its loop).  False: never (too
-// many inputs or dependencies, a far offset, a cycle of waits).
+// An engine's records in one iteration of a loop, fixed loops entered: f(op
+// record's index, record, the control costs since the engine's previous one);
+// returns the costs after the last.
+template <int MODE, class F>
+__device__ __forceinline__ int32_t trip_walk(const SweepArgs& a, const BarProg& b, int row, int e, F f) {
+  const bool elide = a.prm.trip_register_elision != 0;
+  int back[SYNC_MAX_DEPTH + 1];
+  int d = 0;
+  int32_t pre = 0;
+  for (int i = __ldg(a.bar.op_ptr + row + e);;) {
+    const int4 o = __ldg(a.bar.ops + i);
+    if (o.x >= 0) {
+      f(i, o, pre);
+      pre = 0;
+      ++i;
+    } else if (o.x == OP_LOOP) {
+      const int c = b.loop_base + (o.y - b.le_base) / b.ne;
+      const int32_t reg = elide && __ldg(a.lflag + c) ? 0 : a.prm.c_regop;       // r-hat := 0, r-hat++
+      pre += 2 * reg + a.prm.c_regop + a.prm.c_branch + hoist_ops<MODE, false>(a, o.y + e);
+      back[d++] = i + 1;
+      i = __ldg(a.bar.op_ptr + o.y + e);
+    } else {
+      if (d == 0) return pre;
+      i = back[--d];
+    }
+  }
+}
+
+// Builds the map of a loop.  False: never (too many records, inputs or
+// dependencies, a far offset, a cycle of waits).
 template <int MODE>
-__device__ __noinline__ bool trip_build(const SweepArgs& a, int32_t* map, const int4 ch, int ne, int lane) {
-  LaneRec L;
-  load_lane(a, ch, lane, L);
-  const bool have = lane < ch.y;
-  const int e = L.meta.x, head = L.meta.z;
-  const int32_t ii = a.prm.ii, lat = L.rec.y;
-  const int32_t A = have ? wait_ops<MODE>(a, L.rec, L.sr.w) + ii : 0;
-  int32_t* x_of = map + kTripOut;
-  int32_t* sem_of = map + kTripIn;
-  const int32_t sem = have ? L.sr.x : -1;
-  x_of[lane] = have ? L.rec.x : -1;
+__device__ __noinline__ bool trip_build(const SweepArgs& a, int32_t* map, const BarProg b, int loop, int lane) {
+  const int ne = b.ne, row = bar_row(b, loop);
+  // the records, engine by engine
+  int32_t *ids = map + kTripIn, *pres = ids + 32, *engs = ids + 64, *sem_of = ids + 96;
+  int cnt = 0;
+  int32_t tail = 0;
+  if (lane < ne) tail = trip_walk<MODE>(a, b, row, lane, [&](int, const int4&, int32_t) { ++cnt; });
+  int at = cnt;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, at, o);
+    if (lane >= o) at += v;
+  }
+  const int n_rec = __shfl_sync(kFull, at, 31);
+  if (n_rec == 0 || n_rec > 32) return false;
+  at -= cnt;
+  const int first_of = at;
+  if (lane < ne)
+    trip_walk<MODE>(a, b, row, lane, [&](int i, const int4&, int32_t pre) {
+      ids[at] = i;
+      pres[at] = pre;
+      engs[at++] = lane;
+    });
+  map[kTripTail + lane] = tail;
+  __syncwarp();
+  const bool have = lane < n_rec;
+  const int op = have ? ids[lane] : -1, e = have ? engs[lane] : 0;
+  const int head = __shfl_sync(kFull, first_of, e);
+  const int4 rec = have ? __ldg(a.bar.ops + op) : make_int4(0, 0, 0, 0);
+  const int4 sr = have ? __ldg(a.opsem + op) : make_int4(-1, 0, 0, 0);
+  const int32_t ii = a.prm.ii, lat = rec.y;
+  const int32_t A = have ? pres[lane] + wait_ops<MODE>(a, rec, sr.w) + ii : 0;
+  const int32_t sem = sr.x;
+  map[kTripX + lane] = rec.x;
   sem_of[lane] = sem;
   // engine runs and semaphore groups
   const unsigned run = __match_any_sync(kFull, have ? e : 32 + lane), grp = __match_any_sync(kFull, sem >= 0 ? sem : -2 - lane);
@@ -63,7 +119,7 @@ __device__ __noinline__ bool trip_build(const SweepArgs& a, int32_t* map, const 
   map[kTripInc + lane] = sem >= 0 ? sem | __popc(grp & lanemask_le()) << 16 | __popc(grp) << 24 : -1;
   __syncwarp();
   // dependencies, one index each
-  const int z = have ? L.rec.z : 0;
+  const int z = rec.z;
   int pre = z;
   for (int o = 1; o < 32; o <<= 1) {
     const int v = __shfl_up_sync(kFull, pre, o);
@@ -76,18 +132,22 @@ __device__ __noinline__ bool trip_build(const SweepArgs& a, int32_t* map, const 
   uint64_t intra = 0;
   int n_intra = 0;
   for (int j = 0; j < z; ++j) {
-    const int r = L.rec.w + j;
+    const int r = rec.w + j;
     const DepInfo D = a.bar.dep[__ldg(a.bar.ddep + r)];
+    const BarDep bd = a.bar.bdep[r];
     const int32_t s = __ldg(a.dsem + r);
     int kind = TD_OUTER, k = 0, rank = 0, inc = 0, p = 0;
     if (s < 0 || s > 0x7fff) { ok = false; continue; }
-    if (D.up == 0) {                        // carried by this loop: the producer is in the body
-      const int32_t op = a.bar.bdep[r].prod_op, x = op >= 0 ? __ldg(a.bar.ops + op).x : -2;
-      while (p < 32 && x_of[p] != x) ++p;
+    int sl = bd.cons_loop;                  // the common loop S
+    for (int u = 0; u < D.up; ++u) sl = a.loop[sl].parent;
+    const bool body = a.bar.bl[sl].host == loop;
+    // carried at a fixed loop: no wait (one iteration a trip)
+    if (body && (D.k == 0 || sl == loop)) {
+      while (p < n_rec && ids[p] != bd.prod_op) ++p;
       k = D.k;
-      if (p == 32 || k > 3) { ok = false; continue; }
+      if (p == n_rec || k > 3) { ok = false; continue; }
       kind = k == 0 ? TD_CHUNK : TD_CARRIED;
-      for (int i = 0; i < 32; ++i)
+      for (int i = 0; i < n_rec; ++i)
         if (sem_of[i] == s) { ++inc; rank += i <= p; }
       if (kind == TD_CHUNK) {
         if (n_intra == kMaxIntra) { ok = false; continue; }
@@ -96,7 +156,7 @@ __device__ __noinline__ bool trip_build(const SweepArgs& a, int32_t* map, const 
     }
     reinterpret_cast<int64_t*>(map + kTripSeg)[pre + j] = __ldg(a.dseg + r);
     map[kTripR + pre + j] = r;
-    map[kTripDep + pre + j] = kind | k << 2 | rank << 4 | inc << 10 | s << 16;
+    map[kTripDep + pre + j] = kind | k << 2 | rank << 4 | inc << 10 | s << 16 | (body ? 1 << 31 : 0);
     map[kTripCol + pre + j] = lane | p << 8;       // until the columns are known
   }
   if (__ballot_sync(kFull, !ok)) return false;
@@ -129,7 +189,7 @@ __device__ __noinline__ bool trip_build(const SweepArgs& a, int32_t* map, const 
     const int32_t known = kind == TC_CARRIED && lane == to ? 0 : kTripNone;
     int32_t r_intra = kTripNone, issue = kTripNone, retire = kTripNone;
     bool settled = false;
-    for (int pass = 0; pass < ch.y + 2 && !settled; ++pass) {
+    for (int pass = 0; pass < n_rec + 2 && !settled; ++pass) {
       const int32_t ready = max(known, r_intra);
       int32_t Ai = A, Bi = have && ready >= 0 ? ready + ii : kTripNone;
 #pragma unroll
@@ -161,7 +221,7 @@ __device__ __noinline__ bool trip_build(const SweepArgs& a, int32_t* map, const 
   }
   if (lane == 0) {
     map[kTripHead + 1] = col;
-    map[kTripHead + 2] = nd;
+    map[kTripHead + 2] = nd | n_rec << 8;
   }
   __syncwarp();
   return true;
@@ -248,36 +308,37 @@ __device__ __forceinline__ void trip_times(const SweepArgs& a, const WarpSmem& S
   }
 }
 
-// Iterations lo .. hi-1 of a trip by the map of its body's chunk `ch`; the
-// first iteration start has been charged.  Returns the first iteration it
-// did not take (the state is then as that iteration starts).
-// FUSED: the thresholds are computed (walk level lc), and compared with the
-// Eq. (1) minimum if asked; a trip where they differ is walked, which tallies.
+// Iterations lo .. hi-1 of loop `loop` by its map; the first iteration start
+// has been charged.  Returns the first iteration it did not take (the state
+// is then as that iteration starts).  FUSED: the thresholds are computed
+// (walk level lc), and compared with the Eq. (1) minimum if asked; a trip
+// where they differ is walked, which tallies.
 template <int MODE, bool TL, bool FUSED>
-__device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& S, const ProgInfo& pi, const int4 ch,
+__device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& S, const ProgInfo& pi, int loop,
                                             int32_t lo, int32_t hi, int lane, int lc, int32_t iter_cost,
                                             unsigned long long& chk) {
   int32_t* map = S.map;
   const int32_t total = hi - lo;
+  if (total < kTripMin || !map[kTripHead + 4]) return lo;
   const int4 hd = *reinterpret_cast<const int4*>(map + kTripHead);
-  if (total < kTripMin || ch.y == 0 || !map[kTripHead + 4]) return lo;
-  const bool same = hd.x == ch.x;
+  const bool same = hd.x == loop;
   const int32_t walked = same ? hd.w : 0;
-  if (walked < 0) return lo;
-  int nc = hd.y, nd = hd.z;
+  if (walked < 0 || (!same && a.bar.bl[loop].foff >= 0)) return lo;
+  int nc = hd.y, nd = hd.z & 255, n_rec = hd.z >> 8;
   if (!same || nc == 0) {
     __syncwarp();
-    if (lane == 0) *reinterpret_cast<int4*>(map + kTripHead) = make_int4(ch.x, 0, 0, walked + total);
+    if (lane == 0) *reinterpret_cast<int4*>(map + kTripHead) = make_int4(loop, 0, 0, walked + total);
     __syncwarp();
     if (walked < kTripLearn) return lo;
-    if (!trip_build<MODE>(a, map, ch, pi.ne, lane)) {
+    if (!trip_build<MODE>(a, map, bar_prog(pi), loop, lane)) {
       __syncwarp();
-      if (lane == 0) *reinterpret_cast<int4*>(map + kTripHead) = make_int4(ch.x, 0, 0, -1);
+      if (lane == 0) *reinterpret_cast<int4*>(map + kTripHead) = make_int4(loop, 0, 0, -1);
       __syncwarp();
       return lo;
     }
     nc = map[kTripHead + 1];
-    nd = map[kTripHead + 2];
+    nd = map[kTripHead + 2] & 255;
+    n_rec = map[kTripHead + 2] >> 8;
   }
   // the thresholds name the dependencies' own producers: lane d holds
   // dependency d's {segment, first value, step, iterations without}
@@ -289,12 +350,15 @@ __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& 
   if (lane < nd) {
     const int32_t D = map[kTripDep + lane];
     seg = segs[lane] + lo;
-    const int32_t pub = S.semv[D >> 16];
+    const int32_t pub = S.semv[(D >> 16) & 0x7fff];
     dk = (D >> 2) & 3;
     if ((D & 3) == TD_OUTER) {
       if (FUSED) {
-        const DepInfo F = a.dep[__ldg(a.ddep + map[kTripR + lane])];
-        const int2 v = S.lvl[lc - F.up];
+        // (carried at a fixed loop of the body: no wait)
+        const int r = map[kTripR + lane];
+        const DepInfo F = a.dep[__ldg(a.ddep + r)];
+        const int below = a.loop[a.bar.bdep[r].cons_loop].depth - a.loop[loop].depth;   // the consumer's loop
+        const int2 v = D < 0 ? make_int2(lo, lo) : S.lvl[lc + below - F.up];
         T0 = wait_value(a, F, v.x, v.y, MODE);
         bad = a.chk_counts && minimum(a, F, v.x, v.y, MODE) != T0;
       } else {
@@ -315,14 +379,14 @@ __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& 
   if (kind == TC_CURSOR) in = S.t[eng];
   if (kind == TC_RETIRE) in = S.lr[eng];
   if (kind == TC_OUTER && To > 0) {
-    const int s = map[kTripDep + dep] >> 16;
+    const int s = (map[kTripDep + dep] >> 16) & 0x7fff;
     in = S.semv[s] - To <= S.rmask ? S.ring[s * (S.rmask + 1) + ((To - 1) & S.rmask)] : a.hist[S.semhb[s] + (To - 1)];
   }
   int32_t h1 = kTripNone, h2 = kTripNone;
   // this lane's record
   const int rec = map[kTripRec + lane], inc = map[kTripInc + lane];
   int32_t own_pub = 0;
-  if (lane < ch.y) {
+  if (lane < n_rec) {
     int4 P = make_int4(0, 0, 0, -1);
     if (inc >= 0) {
       const int s = inc & 0xffff;
@@ -333,15 +397,16 @@ __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& 
     }
     int4* out = reinterpret_cast<int4*>(map + kTripOut) + 2 * lane;
     out[0] = P;
-    out[1] = make_int4(S.nn[rec & 255] + (rec >> 16), (rec >> 8) & 255, rec & 255, __ldg(a.lrec + ch.x + lane).x);
+    out[1] = make_int4(S.nn[rec & 255] + (rec >> 16), (rec >> 8) & 255, rec & 255, map[kTripX + lane]);
   }
   __syncwarp();
   if (FUSED) {                              // all iterations first: the walk cannot take over in a trip
     for (int d = 0; d < nd; ++d) {
+      if ((map[kTripDep + d] & 3) == TD_OUTER) continue;    // constant over the trip
       const DepInfo F = a.dep[__ldg(a.ddep + map[kTripR + d])];
-      if (F.up > 0) continue;                // constant over the trip
       const int32_t w0 = __shfl_sync(kFull, T0, d), st = __shfl_sync(kFull, step, d);
       for (int32_t j = lane; j < total; j += 32) {
+        // offset 0 may be carried by a fixed loop: the trip's start is then no matter
         const int32_t T = wait_value(a, F, lo + j, lo, MODE);
         bad = bad || T != (j < F.k ? 0 : w0 + j * st) || (a.chk_counts && minimum(a, F, lo + j, lo, MODE) != T);
       }
@@ -368,16 +433,16 @@ __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& 
       }
     }
     if (__ballot_sync(kFull, bad)) break;
-    const int32_t add = a.prm.ii + ic;
+    const int32_t add = a.prm.ii + ic + map[kTripTail + eng];
     if (groups <= 2) trip_inputs<2>(map, lane, kind, from, k, add, nb, in, h1, h2);
     else if (groups == 3) trip_inputs<3>(map, lane, kind, from, k, add, nb, in, h1, h2);
     else if (groups == 4) trip_inputs<4>(map, lane, kind, from, k, add, nb, in, h1, h2);
     else trip_inputs<6>(map, lane, kind, from, k, add, nb, in, h1, h2);
     __syncwarp();
-    if (groups <= 2) trip_times<2, TL>(a, S, map, ch.y, lane, done, nb, lo, chk);
-    else if (groups == 3) trip_times<3, TL>(a, S, map, ch.y, lane, done, nb, lo, chk);
-    else if (groups == 4) trip_times<4, TL>(a, S, map, ch.y, lane, done, nb, lo, chk);
-    else trip_times<6, TL>(a, S, map, ch.y, lane, done, nb, lo, chk);
+    if (groups <= 2) trip_times<2, TL>(a, S, map, n_rec, lane, done, nb, lo, chk);
+    else if (groups == 3) trip_times<3, TL>(a, S, map, n_rec, lane, done, nb, lo, chk);
+    else if (groups == 4) trip_times<4, TL>(a, S, map, n_rec, lane, done, nb, lo, chk);
+    else trip_times<6, TL>(a, S, map, n_rec, lane, done, nb, lo, chk);
     __syncwarp();
   }
   done = min(done, total);
@@ -386,8 +451,9 @@ __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& 
   const unsigned in_body = __reduce_or_sync(kFull, kind == TC_CURSOR ? 1u << eng : 0u);
   if (kind == TC_CURSOR) S.t[eng] = done == total ? in - ic : in;
   if (kind == TC_RETIRE) S.lr[eng] = in;
-  if (lane < pi.ne && !((in_body >> lane) & 1)) S.t[lane] += (done == total ? done - 1 : done) * iter_cost;
-  if (lane < ch.y) {
+  if (lane < pi.ne && !((in_body >> lane) & 1)) 
+    S.t[lane] += (done == total ? done - 1 : done) * iter_cost + done * map[kTripTail + lane];
+  if (lane < n_rec) {
     const int cnt = (rec >> 8) & 255, per = inc >> 24;
     if ((rec >> 16) == cnt) S.nn[rec & 255] += done * cnt;
     if (inc >= 0 && ((inc >> 16) & 255) == per) S.semv[inc & 0xffff] = own_pub + done * per;

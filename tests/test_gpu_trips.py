@@ -50,11 +50,37 @@ def program(trips, records, engines, density, k_max, rng):
     return b.batch()
 
 
+def fixed_program(trips, records, rng):
+    """A loop of conditionals taken always, some nested, beside records of its
+    own, each instruction waiting for the one before it, and a record no
+    engine of the body runs."""
+    b = workloads.ProgramBuilder(5)
+    A = b.loop(0, 0, [len(trips)])
+    L = b.loop(A, 0, trips)
+    n = sum(trips)
+    xs, where = [], L
+    for i in range(records):
+        where = b.loop(L, i, [1] * n) if i % 3 else L
+        if i % 3 == 2:
+            where = b.loop(where, 0, [1] * n)
+        xs.append(b.instr(where, i, int(rng.integers(0, 4)), int(rng.integers(1, 200))))
+    z = b.instr(A, 1, 4, 7)
+    for p, c in zip(xs, xs[1:]):
+        b.dep(p, c, 0)
+    b.dep(xs[-1], xs[0], 1)
+    b.dep(xs[3 * ((records - 1) // 3)], xs[0], 2)
+    b.dep(xs[-1], xs[-1], 1)
+    b.dep(xs[-1], z, 0)
+    b.dep(z, xs[0], 1)
+    return b.batch()
+
+
 def batch_of(rng):
     trips = [[40] + [t, t + 1, 0, 64, t] for t in (1, 3, 4, 31, 32, 33, 65)]
     shapes = [(1, 1, 0.9, 1), (2, 2, 0.9, 3), (5, 3, 0.6, 4), (16, 4, 0.4, 2), (17, 5, 0.3, 3), (32, 8, 0.15, 2),
               (32, 2, 0.8, 2), (31, 12, 0.2, 1)]
-    return workloads.concat([program(t, *s, rng) for t in trips for s in shapes])
+    return workloads.concat([program(t, *s, rng) for t in trips for s in shapes] +
+                            [fixed_program(t, n, rng) for t in trips for n in (1, 2, 7, 20)])
 
 
 @pytest.mark.parametrize("seed", range(2))
