@@ -135,8 +135,10 @@ class ClockSampler:
 KERNEL_SOURCES = {
     "thresholds": ("k_thresholds.cu", "waitval.cuh", "enc.h"),
     "check": ("k_thresholds.cu", "waitval.cuh", "enc.h"),
-    "sim_barrier_free": ("k_sweep.cu", "sweep.cuh", "k_simulate.cu", "cost.cuh", "waitval.cuh", "enc.h"),
-    "sim_barrier": ("k_sweep.cu", "sweep.cuh", "k_simulate.cu", "cost.cuh", "waitval.cuh", "enc.h"),
+    "sim_barrier_free": ("k_sweep.cu", "k_sweep_maps.cu", "sweep.cuh", "trip.cuh", "k_simulate.cu", "cost.cuh",
+                         "waitval.cuh", "enc.h"),
+    "sim_barrier": ("k_sweep.cu", "k_bar.cu", "bar.cuh", "sweep.cuh", "k_simulate.cu", "cost.cuh", "waitval.cuh",
+                    "enc.h"),
 }
 
 

@@ -713,7 +713,9 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   const size_t o_hist = L.add<int32_t>(hist_max), o_slot = L.add<int32_t>(kCounters + (int64_t)P);
   const size_t o_tile_first = L.add<int32_t>(n_first_tiles + 1), o_tile_job = L.add<int32_t>(n_job_tiles + 1);
   const int64_t n_tiles = cnt[BC_TILES];
-  const size_t o_tile_loop = L.add<int32_t>(n_tiles + 1), o_F = L.add<int32_t>(cnt[BC_FPOOL]);
+  // past this the interval starts would crowd out the batch itself: walked
+  const bool bar_fits = cnt[BC_FPOOL] <= kBarPoolMax;
+  const size_t o_tile_loop = L.add<int32_t>(n_tiles + 1), o_F = L.add<int32_t>(bar_fits ? cnt[BC_FPOOL] : 0);
   const size_t o_rel = L.add<int2>(n_ops), o_ko = L.add<int2>(NL), o_bind = L.add<uint8_t>(ND);
   const size_t o_left = L.add<int32_t>(P), o_counted = L.add<int32_t>(P), o_todo = L.add<int32_t>((int64_t)P + 1);
   char* dev = h.alloc<char>((int64_t)L.bytes, "encoding");
@@ -806,7 +808,7 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   h.next_slot = reinterpret_cast<int32_t*>(D(o_slot));
   h.fallback = h.next_slot + kCounters - 1;
   BarArgs& b = h.bar;
-  b.on = div ? 0 : 1;
+  b.on = !div && bar_fits;
   b.n_tiles = (int32_t)n_tiles;
   b.bl = reinterpret_cast<BarLoop*>(D(o_bl));
   b.bdep = reinterpret_cast<BarDep*>(D(o_bdep));

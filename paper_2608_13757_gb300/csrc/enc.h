@@ -350,6 +350,7 @@ constexpr int32_t kBarBad = 1 << 30;
 // by intervals).
 constexpr int32_t kBarMinInst = 256;
 constexpr size_t kBarRingBytes = 32 * 1024;
+constexpr int64_t kBarPoolMax = int64_t(8) << 30;   // entries of F: 32 GB
 // Counters a sweep launch starts from, zeroed together: next_slot[0], the
 // intervals' count of planned programs, fallback[0] (the list follows).
 constexpr int32_t kCounters = 3;

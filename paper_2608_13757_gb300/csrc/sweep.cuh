@@ -23,6 +23,9 @@
 //     cycle never settles and is a deadlock);
 //   - a threshold beyond every increment up to this chunk points forward in
 //     program order: the program is handed to the per-engine kernel.
+// Trips of loops around straight lines go by their max-plus maps where that
+// pays (trip.cuh, sweep_maps in enc.h); the barrier scheme by intervals
+// (bar.cuh), its walk only for what those leave.
 // A loop whose body is one chunk runs all its iterations in a tight loop
 // with the lanes' records in registers and the next iteration's thresholds
 // in flight.  Barriers (barrier scheme) are a warp maximum of the engines'
