@@ -472,7 +472,8 @@ __device__ __forceinline__ bool bar_waits(const SweepArgs& a, const BarProg& b, 
     for (int k = 0; k < n; ++k) {
       const int kk = __shfl_sync(kBarFull, kind, k);
       const int64_t so = __shfl_sync(kBarFull, seg, k);
-      if (FUSED || MODE == SYNC_THR_PERENGINE || (kk & 3) == 3) {
+      // (thresholds that start off a 16-byte boundary are read one by one)
+      if (FUSED || MODE == SYNC_THR_PERENGINE || (kk & 3) == 3 || (reinterpret_cast<uintptr_t>(a.thr) & 15)) {
         const int rr = __shfl_sync(kBarFull, r, k);
         const DepInfo D = a.bar.dep[__ldg(a.bar.ddep + rr)];
         const BarDep bd = a.bar.bdep[rr];

@@ -481,14 +481,15 @@ T* sized(HostVec<T>& v, int64_t n) {
 class Team {
  public:
   explicit Team(int n) {
+    err_.resize(n);
+    pool_.reserve(n);
     for (int t = 1; t < n; ++t) {
       try {
         pool_.emplace_back([this, t] { work(t); });
-      } catch (const std::system_error&) {
+      } catch (...) {
         break;
       }
     }
-    err_.resize(pool_.size() + 1);
   }
   ~Team() {
     {

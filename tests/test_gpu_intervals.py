@@ -96,3 +96,25 @@ def test_waits_that_do_not_repeat(sg, mode):
     assert np.array_equal(r.checksum.cpu().numpy()[:P].view(np.uint64), ref.checksum)
     assert (ref.status == 0).any() and (ref.status != 0).any()
     h.close()
+
+
+@pytest.mark.parametrize("mode", ALL_MODES)
+@pytest.mark.parametrize("at", [1, 2, 3])
+def test_thresholds_off_a_16_byte_boundary(sg, mode, at):
+    """A threshold array that starts anywhere in a larger one."""
+    import torch
+    rng = np.random.default_rng(5)
+    batch = workloads.concat([program(total, 7, 9, 0.2, rng) for total in (1, 33, 129, 513)])
+    h = sg.sync_load_programs(batch)
+    thr = sg.sync_eval_thresholds(h, mode)
+    buf = torch.full((thr.numel() + 8,), 1 << 20, dtype=torch.int32, device=thr.device)
+    off = buf[at:at + thr.numel()]
+    off.copy_(thr)
+    assert off.data_ptr() % 16 == 4 * at
+    for variant in (oracle.BARRIER, oracle.BARRIER_FREE):
+        want = sg.sync_simulate(h, mode, thr, variant=variant)
+        got = sg.sync_simulate(h, mode, off, variant=variant)
+        for f in ("status", "makespan", "checksum"):
+            assert torch.equal(getattr(got, f), getattr(want, f))
+        assert not want.status.any()
+    h.close()
