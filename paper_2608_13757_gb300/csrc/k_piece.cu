@@ -296,18 +296,12 @@ __global__ void __launch_bounds__(kValThreads) k_piece_fixup(const SweepArgs a, 
 template <class K>
 cudaError_t launch_items(K kern, const SweepArgs& a, int64_t items, size_t smem, int num_sms, cudaStream_t s) {
   if (items <= 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  SweepShape sh;
+  cudaError_t e = sweep_shape(kern, items, smem, num_sms, true, sh);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const long long want = (items + kWarps - 1) / kWarps;
-  const long long cap = (long long)num_sms * per_sm;
-  const int grid = (int)(want < cap ? want : cap);
   e = cudaMemsetAsync(a.next_slot, 0, sizeof(int32_t), s);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kWarps * 32, smem, s>>>(a);
+  kern<<<sh.grid, sh.threads, sh.smem, s>>>(a);
   return launched();
 }
 

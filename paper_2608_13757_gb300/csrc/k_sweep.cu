@@ -8,10 +8,12 @@ namespace {
 template <int MODE, bool BB>
 cudaError_t launch3(const SweepArgs& a, size_t smem, int num_sms, cudaStream_t s) {
   long long items = a.n_programs;
-  auto run = [&](auto kern) { return run_sweep(kern, a, items, smem, num_sms, s); };
+  bool spread = true;
+  auto run = [&](auto kern) { return run_sweep(kern, a, items, smem, num_sms, s, spread); };
   if constexpr (BB) {
     if (a.bar.on && a.bar.n_tiles > items) items = a.bar.n_tiles;
     if (a.bar.on || a.bar.todo) {
+      spread = false;                          // tiles are dealt out kWarps a CTA
       if (a.dep)
         return a.issue ? run(k_sweep<MODE, true, true, true, false, true>) : run(k_sweep<MODE, true, false, true, false, true>);
       return a.issue ? run(k_sweep<MODE, true, true, false, false, true>) : run(k_sweep<MODE, true, false, false, false, true>);

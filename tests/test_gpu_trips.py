@@ -118,3 +118,11 @@ def test_waits_on_other_increments(sg, mode):
     assert np.array_equal(r.checksum.cpu().numpy()[:P].view(np.uint64), ref.checksum)
     assert (ref.status == 0).any() and (ref.status != 0).any()
     h.close()
+
+
+@pytest.mark.parametrize("config", ["syncbound", "small"])
+@pytest.mark.parametrize("programs", [1, 7, 151, 152, 153, 305, 1216, 1217, 1368, 2433, 3649])
+def test_programs_over_the_sms(sg, config, programs):
+    """Batches around a warp, 8 warps and whole CTAs on every SM, whose
+    sweeps take CTAs of 1 to 8 warps."""
+    compare_all(sg, workloads.generate(config, n_programs=programs), modes=[oracle.PERLOOP])
