@@ -318,8 +318,14 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
     p.pcs.spec = 0;
     p.ring = sweep_ring(p.sem_cap, p.frame_depth, false);
     const size_t smem = sweep_smem_bytes(p.sem_cap, p.frame_depth, p.ring, false);
-    e = launch_items(k_sweep<MODE, false, true, false, true>, p, (int64_t)p.pcs.n_pieces * p.pcs.probes, smem,
-                     num_sms, s);
+    // 128 registers a thread (no spills) and 16 warps per SM, unless 24 warps
+    // take all runs at once and 16 do not: GEMM batches at 80 / 128
+    // registers, 1 program (320 runs) 2.30 / 2.14 ms, 4 3.20 / 3.05, 8 (2560)
+    // 6.1 / 7.4, 12 (3840) 10.9 / 8.5, 20 15.3 / 13.7.
+    const int64_t runs = (int64_t)p.pcs.n_pieces * p.pcs.probes;
+    const bool one_wave = runs > 2 * kWarps * num_sms && runs <= 3 * kWarps * num_sms;
+    e = one_wave ? launch_items(k_sweep<MODE, false, true, false, true>, p, runs, smem, num_sms, s)
+                 : launch_items(k_sweep<MODE, false, true, false, true, false, false, true>, p, runs, smem, num_sms, s);
     if (e != cudaSuccess) return e;
     k_piece_resolve<<<warp_blocks, 256, 0, s>>>(p, L.n_split);
     if ((e = launched()) != cudaSuccess) return e;

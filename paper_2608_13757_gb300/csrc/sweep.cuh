@@ -887,9 +887,9 @@ __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, c
 // start and ends after its last iteration.
 // BAR (barrier scheme): programs by intervals (bar.cuh), and by the walk only
 // those the intervals leave.  MAPS (barrier-free): trips by their maps
-// (trip.cuh).
-template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false, bool BAR = false, bool MAPS = false>
-__global__ void __launch_bounds__(kWarps * 32, MAPS ? 2 : BAR ? kBarCtas : 3) k_sweep(const __grid_constant__ SweepArgs a) {
+// (trip.cuh).  REGS: 128 registers and 16 warps per SM without maps.
+template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false, bool BAR = false, bool MAPS = false, bool REGS = false>
+__global__ void __launch_bounds__(kWarps * 32, MAPS || REGS ? 2 : BAR ? kBarCtas : 3) k_sweep(const __grid_constant__ SweepArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   WarpSmem S;

@@ -160,3 +160,9 @@ def test_kernel_launch_count(sg, spec, monkeypatch):
         else:
             assert bf in (2 + 1 + 2 + 1, 2 + 1 + 2 + 9 + 1, 2 + 1 + 9 + 1)
         h.close()
+
+
+@pytest.mark.parametrize("programs", [2, 8])
+def test_probed_pieces_either_kernel(sg, programs):
+    """Probe runs that fit 16 warps per SM, and that fit 24 but not 16."""
+    compare_all(sg, workloads.generate("gemm", n_programs=programs), modes=[oracle.PERLOOP])
