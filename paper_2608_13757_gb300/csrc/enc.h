@@ -294,7 +294,7 @@ struct alignas(16) BarLoop {   // per loop, and a last entry (tile0: all tiles)
   int32_t prog;
   int32_t item;      // its plan item in its parent's body
   int32_t host;      // itself unless fixed
-  int32_t nchild;    // child loops that are not fixed
+  int32_t fbar;      // 1: a barrier-fallback barrier ends its iterations, or those of a fixed loop in them
   int32_t esib;      // such loops before it in its parent's body
   int32_t tile0;     // its first tile
   int32_t iters;     // iterations per tile (a multiple of 32)

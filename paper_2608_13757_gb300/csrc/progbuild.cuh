@@ -823,7 +823,7 @@ struct ProgBuilder {
       BarLoop& b = O.bl[l0 + l];
       b.foff = nchild > 0 ? c[BC_FPOOL] : -1;
       b.prog = p;
-      b.nchild = nchild;
+      b.fbar = S.fbar[l0 + l];
       b.tile0 = (int32_t)c[BC_TILES];
       b.iters = iters;
     }
@@ -957,6 +957,8 @@ struct ProgBuilder {
       }
       c[BC_OPS] = at;
     }
+    for (int32_t l = nl - 1; l > 0; --l)        // a fixed loop's barriers are in its host's iterations
+      if (fixed(l) && O.bl[l0 + l].fbar) O.bl[l0 + par[l]].fbar = 1;
   }
 
   // one sweep chunk: n <= 32 lanes `recs` (program-local instructions,

@@ -2,7 +2,8 @@
 // for loops whose iterations are one straight line of at most 32 records: no
 // child loops but fixed ones (which run exactly once on every visit, so
 // their records' instances are the loop's iterations and they cost every
-// engine the same each time).
+// engine the same each time), and no barrier-fallback barrier, which joins
+// the engines and is no record.
 //
 // With its waits inside an iteration fixed, every issue and retire of an iteration is a
 // maximum, over the engines' cursors and last retires at its start and the
@@ -328,7 +329,7 @@ __device__ __forceinline__ int32_t run_trip(const SweepArgs& a, const WarpSmem& 
   const int4 hd = *reinterpret_cast<const int4*>(map + kTripHead);
   const bool same = hd.x == loop;
   const int32_t walked = same ? hd.w : 0;
-  if (walked < 0 || (!same && a.bar.bl[loop].foff >= 0)) return lo;
+  if (walked < 0 || (!same && (a.bar.bl[loop].foff >= 0 || a.bar.bl[loop].fbar))) return lo;
   int nc = hd.y, nd = hd.z & 255, n_rec = hd.z >> 8;
   if (!same || nc == 0) {
     __syncwarp();

@@ -181,3 +181,89 @@ def test_fallback_loader_offsets(sg):
     assert_parts_match(sg, b, [0, 45, 90, 102, 172], (COUNT, PERLOOP, PERENGINE),
                        (sg.SIM_BARRIER_FREE, sg.SIM_BARRIER))
 
+
+
+def flagged_program(kind, backward, trips=(40, 40, 40), lat=50):
+    """Loops of long trips around loops that run once on every visit, with a
+    fallback barrier at the outer loop ("host"), at a loop that itself runs
+    once ("fixed"), or at both."""
+    pb, n = workloads.ProgramBuilder(2), sum(trips)
+    a = pb.loop(0, 0, [len(trips)])
+    h = pb.loop(a, 0, list(trips))
+    s = h if kind == "host" else pb.loop(h, 1, [1] * n)
+    c = pb.loop(s, 1, [1] * n)
+    p = pb.instr(c, 0, engine=0, latency=lat)
+    at = 0 if backward else 2
+    pb.dep(p, pb.instr(s, at, engine=1, latency=3), 2)
+    if kind == "both":
+        pb.dep(p, pb.instr(h, at, engine=1, latency=5), 2)
+    return pb.batch()
+
+
+def random_flagged(rng):
+    """A loop of trips 20 to 60 around a random tree of loops that mostly run
+    once, instructions waiting for earlier ones and, at offsets 0 to 3, for
+    those of the loops below theirs."""
+    engines = int(rng.integers(2, 6))
+    pb = workloads.ProgramBuilder(engines)
+    trips = rng.integers(20, 61, size=3).tolist()
+    a = pb.loop(0, 0, [3])
+    host = pb.loop(a, 0, trips)
+    parent, pos, items, count = {host: a}, {host: 0}, {host: 0}, {host: sum(trips)}
+    inner = []
+    for _ in range(int(rng.integers(1, 5))):
+        up = int(rng.choice([host] + inner))
+        t = [1] * count[up] if rng.random() < 0.8 else rng.integers(0, 3, size=count[up]).tolist()
+        l = pb.loop(up, 3 * items[up] + 1, t)
+        parent[l], pos[l], items[l], count[l] = up, 3 * items[up] + 1, 0, sum(t)
+        items[up] += 1
+        inner.append(l)
+    xs = [(pb.instr(l, 3 * i + d, int(rng.integers(0, engines)), int(rng.integers(1, 90))), l, 3 * i + d)
+          for l in [host] + inner for i in range(items[l] + 1) for d in (0, 2) if rng.random() < 0.7]
+    for c, lc, at in xs:
+        for p, lp, ap in xs:
+            child, l = None, lp
+            while l != lc and l != a:
+                child, l = l, parent[l]
+            if l != lc or rng.random() > 0.25:
+                continue
+            forward = at > (ap if child is None else pos[child])
+            if p != c:
+                pb.dep(p, c, int(rng.integers(0 if forward else 1, 4)))
+    return pb.batch()
+
+
+@pytest.mark.parametrize("beside", [False, True], ids=["alone", "beside_mapped"])
+def test_fallback_in_long_trips(sg, beside):
+    """Barriers at the end of iterations that a trip map would otherwise take
+    (a loop whose child loops all run once), alone and in a batch whose sweep
+    takes trips by maps; also through the call that allocates nothing."""
+    import torch
+    from tests.test_gpu_trips import fixed_program
+    rng = np.random.default_rng(77)
+    parts = [flagged_program(k, bwd) for k in ("host", "fixed", "both") for bwd in (False, True)]
+    parts += [random_flagged(rng) for _ in range(40)]
+    if beside:
+        parts += [fixed_program([64] * 40, 7, rng) for _ in range(12)]
+    b = with_policy(workloads.concat(parts), 1)
+    assert (oracle.classify(b).kase == oracle.CASE_BARRIER).sum() > 40
+    for prm in (oracle.sim_params(), oracle.sim_params(ii=2, c_branch=3, c_regop=2, c_barrier=17, licm=1, cse=1)):
+        h = compare_fallback(sg, b, prm)
+    for mode in (COUNT, PERLOOP, PERENGINE):
+        thr = sg.sync_eval_thresholds(h, mode)
+        want = sg.sync_simulate(h, mode, thr, timeline=True)
+        got = sg.sync_simulate_noalloc(h, mode, thr, timeline=True)
+        for f in ("status", "makespan", "checksum", "issue", "retire"):
+            assert torch.equal(getattr(got, f), getattr(want, f)), (mode, f)
+    h.close()
+
+
+def test_fallback_hand_long_trips(sg):
+    """Three trips of 40 iterations, each ended by a barrier after the
+    producer's 50 cycles: 10693 cycles (1022 without the dependency)."""
+    h = sg.sync_load_programs(with_policy(flagged_program("host", False), 1))
+    thr, _ = gpu_thresholds(sg, h, COUNT)
+    for r in (sg.sync_simulate(h, COUNT, thr), sg.sync_simulate_noalloc(h, COUNT, thr),
+              sg.sync_simulate_fused(h, COUNT)):
+        assert r.status.cpu().tolist()[:1] == [0] and r.makespan.cpu().tolist()[:1] == [10693]
+    h.close()
