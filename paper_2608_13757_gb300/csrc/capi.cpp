@@ -1128,9 +1128,8 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
     a.dep = h->dep; a.ddep = h->ddep; a.path = h->path; a.ord = h->ord;
     a.chk_counts = d_counts; a.chk_first = reinterpret_cast<unsigned long long*>(d_first_bad);
   }
-  const bool maps = variant != SYNC_SIM_BARRIER &&
-                    sweep_maps(h->sz.n_programs, h->sz.n_instances, h->n_stmt, h->num_sms);
-  const int ring = sweep_ring(a.sem_cap, a.frame_depth, maps);
+  bool maps;
+  const int ring = h->sweep_choice(variant, a.sem_cap, a.frame_depth, maps);
   if (simulate_smem_bytes(a.warps, a.sem_cap, a.frame_depth) > 200 * 1024 || ring == 0)
     raise(SYNC_ERR_ARG, "a program has too many waited semaphores for the simulator's shared memory");
   SweepArgs w;

@@ -130,6 +130,15 @@ struct sync_programs {
   // the handle makes its own stream wait for it
   cudaEvent_t ready = nullptr;
 
+  // Whether a simulation's sweep takes trips by their maps, and its ring (0:
+  // none fits).  The maps' shared memory leaves room for up to 240 waited
+  // semaphores, the walk's for 448: past the former the batch is walked.
+  int sweep_choice(sync_sim_variant variant, int32_t sem_cap, int32_t frame_depth, bool& maps) const {
+    maps = variant != SYNC_SIM_BARRIER && syncgb::sweep_maps(sz.n_programs, sz.n_instances, n_stmt, num_sms) &&
+           syncgb::sweep_ring(sem_cap, frame_depth, true) > 0;
+    return syncgb::sweep_ring(sem_cap, frame_depth, maps);
+  }
+
   cudaError_t wait_ready(cudaStream_t s) const { return ready ? cudaStreamWaitEvent(s, ready, 0) : cudaSuccess; }
 
   ~sync_programs() {

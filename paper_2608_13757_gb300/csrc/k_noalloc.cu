@@ -77,9 +77,8 @@ extern "C" sync_status sync_simulate_noalloc(const sync_programs* h, sync_thr_mo
                                    " (use sync_simulate)");
   const int32_t sem_cap = std::max(4, (h->nsem_max[mode] + 3) & ~3);
   const int32_t frame_depth = std::max(1, h->depth_max);
-  const bool maps = variant != SYNC_SIM_BARRIER &&
-                    sweep_maps(h->sz.n_programs, h->sz.n_instances, h->n_stmt, h->num_sms);
-  const int ring = sweep_ring(sem_cap, frame_depth, maps);
+  bool maps;
+  const int ring = h->sweep_choice(variant, sem_cap, frame_depth, maps);
   if (simulate_smem_bytes(h->ne_max, sem_cap, frame_depth) > 200 * 1024 || ring == 0)
     return set_error(SYNC_ERR_ARG, "a program has too many waited semaphores for the simulator's shared memory");
   sync_status st = cuda_error(cudaSetDevice(h->device), "cudaSetDevice");

@@ -317,6 +317,7 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
     SweepArgs p = a;
     p.pcs.spec = 0;
     p.ring = sweep_ring(p.sem_cap, p.frame_depth, false);
+    if (p.ring < 1) return cudaErrorInvalidConfiguration;
     const size_t smem = sweep_smem_bytes(p.sem_cap, p.frame_depth, p.ring, false);
     // 128 registers a thread (no spills) and 16 warps per SM, unless 24 warps
     // take all runs at once and 16 do not: GEMM batches at 80 / 128
@@ -334,15 +335,20 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
   if (L.n_spec > 0) {
     SweepArgs p = a;
     p.pcs.spec = 1;
+    // walked where no ring fits beside the maps (the caller's fits without)
     p.ring = sweep_ring(p.sem_cap, p.frame_depth, true);
-    const size_t smem = sweep_smem_bytes(p.sem_cap, p.frame_depth, p.ring, true);
+    const bool maps = p.ring > 0;
+    if (!maps) p.ring = sweep_ring(p.sem_cap, p.frame_depth, false);
+    if (p.ring < 1) return cudaErrorInvalidConfiguration;
+    const size_t smem = sweep_smem_bytes(p.sem_cap, p.frame_depth, p.ring, maps);
     p.pcs.probes = 1;
     p.pcs.ptimes = L.one;
     p.pcs.plen = L.one_len;
     k_spec_init<<<warp_blocks, 256, 0, s>>>(p, L.n_split);
     if ((e = launched()) != cudaSuccess) return e;
     for (int r = 0; r < kSpecRounds; ++r) {
-      e = launch_items(k_sweep<MODE, false, true, false, true, false, true>, p, p.pcs.n_pieces, smem, num_sms, s);
+      e = maps ? launch_items(k_sweep<MODE, false, true, false, true, false, true>, p, p.pcs.n_pieces, smem, num_sms, s)
+               : launch_items(k_sweep<MODE, false, true, false, true>, p, p.pcs.n_pieces, smem, num_sms, s);
       if (e != cudaSuccess) return e;
       k_spec_resolve<<<warp_blocks, 256, 0, s>>>(p, L.n_split, r == kSpecRounds - 1);
       if ((e = launched()) != cudaSuccess) return e;

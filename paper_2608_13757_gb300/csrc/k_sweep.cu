@@ -42,6 +42,7 @@ int sweep_ring(int sem_cap, int frame_depth, bool maps) {
 
 cudaError_t launch_sweep(const SweepArgs& a, bool barrier, int num_sms, cudaStream_t s) {
   if (a.n_programs == 0) return cudaSuccess;
+  if (a.ring < 1) return cudaErrorInvalidConfiguration;
   if (a.maps) return launch_sweep_maps(a, num_sms, s);
   const size_t smem = sweep_smem_bytes(a.sem_cap, a.frame_depth, a.ring, false);
   if (a.mode == SYNC_THR_PERLOOP)

@@ -166,3 +166,18 @@ def test_kernel_launch_count(sg, spec, monkeypatch):
 def test_probed_pieces_either_kernel(sg, programs):
     """Probe runs that fit 16 warps per SM, and that fit 24 but not 16."""
     compare_all(sg, workloads.generate("gemm", n_programs=programs), modes=[oracle.PERLOOP])
+
+
+@pytest.mark.parametrize("spec", ["0", "1"], ids=["probes", "speculation"])
+@pytest.mark.parametrize("waited", [28, 240, 244, 245, 320, 440])
+def test_pieces_with_many_waited_semaphores(sg, waited, spec, monkeypatch):
+    """Numbers of semaphores that leave a small ring beside the trip maps of
+    speculated pieces, and none."""
+    from tests.test_gpu_trips import many_waits
+    monkeypatch.setenv("SYNCGB_SPLIT_MIN", "1")
+    monkeypatch.setenv("SYNCGB_SPLIT_SPEC", spec)
+    batch = many_waits(waited, 6, np.random.default_rng(waited))
+    h = sg.sync_load_programs(batch)
+    assert h.sizes.n_split_programs == 1
+    h.close()
+    compare_all(sg, batch, timeline=True, modes=[oracle.COUNT])

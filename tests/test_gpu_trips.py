@@ -126,3 +126,41 @@ def test_programs_over_the_sms(sg, config, programs):
     """Batches around a warp, 8 warps and whole CTAs on every SM, whose
     sweeps take CTAs of 1 to 8 warps."""
     compare_all(sg, workloads.generate(config, n_programs=programs), modes=[oracle.PERLOOP])
+
+
+def many_waits(waited, reps, rng):
+    """A loop of `reps` iterations around `waited` producers, each waited on
+    by a consumer of its own, beside a leaf loop of long trips."""
+    b = workloads.ProgramBuilder(4)
+    A = b.loop(0, 0, [reps])
+    for i in range(waited - 1):
+        p = b.instr(A, 2 * i, i % 3, int(rng.integers(1, 50)))
+        b.dep(p, b.instr(A, 2 * i + 1, 3, 2), 0)
+    L = b.loop(A, 2 * waited, [64] * reps)
+    xs = [b.instr(L, i, i % 2, int(rng.integers(1, 50))) for i in range(9)]
+    b.dep(xs[0], xs[1], 0)
+    return b.batch()
+
+
+@pytest.mark.parametrize("waited", [24, 28, 32, 239, 240, 241, 244, 245, 320, 321, 440])
+def test_many_waited_semaphores(sg, waited):
+    """Rings of fewer increments, maps on fewer CTAs, and numbers of
+    semaphores that leave no ring beside the maps, in batches whose sweep
+    takes maps otherwise; also through the call that allocates nothing."""
+    import torch
+    rng = np.random.default_rng(waited)
+    batch = workloads.concat([many_waits(waited, 20, rng)] + [program([70] * 40, 17, 5, 0.3, 2, rng) for _ in range(8)])
+    h = compare_all(sg, batch, modes=[oracle.COUNT])
+    thr = sg.sync_eval_thresholds(h, oracle.COUNT)
+    want, got = sg.sync_simulate(h, oracle.COUNT, thr), sg.sync_simulate_noalloc(h, oracle.COUNT, thr)
+    for f in ("status", "makespan", "checksum"):
+        assert torch.equal(getattr(got, f), getattr(want, f))
+
+
+def test_too_many_waited_semaphores(sg):
+    h = sg.sync_load_programs(many_waits(460, 20, np.random.default_rng(1)))
+    thr = sg.sync_eval_thresholds(h, oracle.COUNT)
+    for call in (sg.sync_simulate, sg.sync_simulate_noalloc):
+        with pytest.raises(sg.SyncError) as err:
+            call(h, oracle.COUNT, thr)
+        assert err.value.status == sg.ERR_ARG
