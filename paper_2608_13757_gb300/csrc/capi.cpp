@@ -218,6 +218,17 @@ void check_totals(const int64_t* count) {
 
 }  // namespace
 
+// A program of `items` equal pieces (1: whole) in a batch's barrier-free cost.
+static void add_cost(SweepCost& c, const ProgSummary& s, int64_t items) {
+  c.walk_max = std::max(c.walk_max, s.walk / items);
+  c.map_max = std::max(c.map_max, s.map / items);
+  c.walk += s.walk;
+  c.map += s.map;
+  c.items += items;
+  c.n_inst += s.n_inst;
+  for (int k = 0; k < 2; ++k) c.n_stmt[k] += s.n_stmt[k];
+}
+
 // Fewest instances of a program cut into pieces: 65536 (SYNCGB_SPLIT_MIN=n
 // sets another floor; tests lower it).
 static int64_t split_floor() {
@@ -239,7 +250,8 @@ static int64_t split_floor() {
 // otherwise (SYNCGB_SPLIT_SPEC=1 speculates always).
 static void build_pieces(const sync_batch_desc& d, const LoopInfo* loop, const int32_t* rowptr, const int4* xsem,
                          const DepInfo* dep, const int64_t* seg, const int64_t* semhb, const ProgInfo* prog,
-                         const int64_t* inst_off, int64_t n_inst, cudaStream_t stream, sync_programs& h) {
+                         const int64_t* inst_off, int64_t n_inst, const ProgSummary* sum, cudaStream_t stream,
+                         sync_programs& h) {
   const int32_t P = d.n_programs;
   const int64_t NX = d.prog_instr_ptr[P];
   const double share = (double)n_inst / ((double)h.num_sms * 24.0);
@@ -346,6 +358,7 @@ static void build_pieces(const sync_batch_desc& d, const LoopInfo* loop, const i
     const bool bf = !force_spec && (double)pi.n_inst > 4.0 * (2.0 * pi.ne + 1.0) * share;
     bf_init.push_back(bf ? 0 : 1);
     if (bf) ne_max = std::max(ne_max, pi.ne);
+    else add_cost(h.spec_cost, sum[p], np);
     // the program's instances in the compact scratch of the stored times
     const int64_t first = nx > 0 ? inst_off[x0] : 0;
     for (int32_t j = 0; j < np; ++j) {
@@ -843,7 +856,7 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
     code_unrolled += s.code_unrolled;
     n_bar_deps += s.n_bar_deps;
     h.max_inst = std::max(h.max_inst, s.n_inst);
-    for (int k = 0; k < 2; ++k) h.n_stmt[k] += s.n_stmt[k];
+    add_cost(h.sweep_cost, s, 1);
     ne_max = std::max(ne_max, s.ne);
     depth_max = std::max(depth_max, s.depth_max);
     ord_overflow |= s.ord_overflow;
@@ -884,7 +897,8 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
     for (int32_t p = 0; p < P && !any; ++p)
       any = a.sum[p].splittable && a.sum[p].n_inst >= min_inst && (double)a.sum[p].n_inst > 8.0 * share;
     if (any)
-      build_pieces(d, O.loop, O.rowptr, O.xsem, O.dep, O.seg, O.semhb, O.prog, O.inst_off, cnt[BC_INST], stream, h);
+      build_pieces(d, O.loop, O.rowptr, O.xsem, O.dep, O.seg, O.semhb, O.prog, O.inst_off, cnt[BC_INST], a.sum,
+                   stream, h);
   }
 
   // ----------------------------------------------------------- device
@@ -911,6 +925,29 @@ static void validate(const sync_batch_desc& d) {
   count_pass(d, sh, team, *SL.s, a, tot);
 }
 
+// For the tests of the dispatch (not part of the interface, no CUDA call):
+// whether a barrier-free simulation of the batch, with at most `waited`
+// semaphores waited on in a program, takes trips by their maps on a GPU of
+// num_sms SMs; -1 for a batch that does not load.
+extern "C" int syncgb_takes_maps(const sync_batch_desc* desc, int num_sms, int waited) {
+  try {
+    const Shape sh = shape_checks(*desc);
+    ScratchLease SL;
+    BuildArgs a{};
+    int64_t tot[kBuildCounts];
+    Team team(load_threads(sh.covered));
+    count_pass(*desc, sh, team, *SL.s, a, tot);
+    SweepCost c{};
+    int depth = 1;
+    for (int32_t p = 0; p < sh.P; ++p) {
+      add_cost(c, a.sum[p], 1);
+      depth = std::max(depth, (int)a.sum[p].depth_max);
+    }
+    return sweep_maps(c, num_sms, std::max(4, (waited + 3) & ~3), depth);
+  } catch (...) {
+    return -1;
+  }
+}
 
 extern "C" {
 
@@ -1175,7 +1212,8 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
     w.pcs.cls = h->piece_cls; w.pcs.need = h->spec_need; w.pcs.has = h->spec_has; w.pcs.xhat = h->spec_xhat;
     w.pcs.shift = h->piece_shift; w.pcs.vp = h->spec_vp;
     SweepArgs wp = w;
-    PieceLaunch L{h->vdep, h->piece_cnt, stored_times(h, true), h->pinst[0], h->n_split, h->n_probed, h->n_spec};
+    PieceLaunch L{h->vdep, h->piece_cnt, stored_times(h, true), h->pinst[0], h->n_split, h->n_probed, h->n_spec,
+                  h->spec_cost};
     wp.pcs.probes = h->probes_bf;
     if (h->n_probed > 0) {                         // the probes' histories and stored times
       wp.pcs.phist = probe_history(h, mode);

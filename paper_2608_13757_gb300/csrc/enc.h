@@ -481,19 +481,21 @@ cudaError_t launch_simulate(const SimArgs& a, bool barrier, int num_sms, cudaStr
 cudaError_t launch_sweep(const SweepArgs& a, bool barrier, int num_sms, cudaStream_t s);
 size_t sweep_smem_bytes(int sem_cap, int frame_depth, int ring, bool maps);
 cudaError_t launch_sweep_maps(const SweepArgs& a, int num_sms, cudaStream_t s);
-// Whether the barrier-free sweep of a batch takes its loops' trips by their
-// maps (trip.cuh; 16 warps per SM instead of 24): where the longest programs
-// bound it, where trips hold most of the work, and where most statements are
-// of fixed loops, which a map takes with their host's iterations.  Instances
-// per statement (not fixed), programs, walked / by maps: chain 264, 4864
-// programs 12.7 / 8.0 ms, 8192 12.9 / 9.5, 16384 14.5 / 14.6, 32768 16.4 /
-// 21.3; depth2 540, 16384 6.9 / 4.5; attention 393, 500 94 / 29; branching
-// trees 20, 6000 0.86 / 1.38; conditionals around one instruction (24 fixed
-// statements to a moving one) 65536 34.0 / 12.5.
-inline bool sweep_maps(int32_t n_programs, int64_t n_instances, const int64_t (&n_stmt)[2], int num_sms) {
-  return n_stmt[1] >= 4 * n_stmt[0] ||
-         (n_instances >= 32 * n_stmt[0] && (n_programs <= 80 * num_sms || n_instances >= 320 * n_stmt[0]));
-}
+// Limits of a trip map (trip.cuh).
+constexpr int kTripCols = 24;               // inputs
+constexpr int kTripMin = 4;                 // shorter trips are walked
+constexpr int kTripLearn = 16;              // iterations walked before a loop's map is built
+// Barrier-free, what a batch's items (programs, or pieces of programs) take
+// one warp with few neighbours, walked and with trips by their maps
+// (sweep_cost in progbuild.cuh): cycles of the longest and of all, items,
+// instances and loop statements of loops that are not fixed and of fixed ones.
+struct SweepCost {
+  int64_t walk_max, map_max, walk, map, items, n_inst, n_stmt[2];
+};
+// Whether a barrier-free sweep takes trips by their maps (k_sweep.cu has the
+// rule), for the batch's largest number of waited semaphores and depth; false
+// also where the maps leave no shared memory for a ring.
+bool sweep_maps(const SweepCost& c, int num_sms, int sem_cap, int frame_depth);
 // Piece-parallel simulation of the split programs (a.pcs), barrier-free:
 // validation, the probe runs or speculation, the composition of the pieces, and the pass that forms the instances' true times (checksums,
 // timelines); the programs it completes are marked in a.pcs.fail (0) for
@@ -504,6 +506,7 @@ struct PieceLaunch {
   int32_t* one;              // stored times of single runs (speculation)
   int64_t one_len;           // instances of all split programs
   int32_t n_split, n_probed, n_spec;   // split programs; of these barrier-free probed / speculated
+  SweepCost spec_cost;       // of the speculated pieces
 };
 cudaError_t launch_pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaStream_t s);
 // Barrier scheme by intervals in separate launches, for a batch with split
@@ -511,7 +514,7 @@ cudaError_t launch_pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms,
 // cannot do are listed in todo for launch_sweep.
 cudaError_t launch_intervals(const SweepArgs& a, int32_t* todo, int32_t n_loops, cudaStream_t s);
 // Largest ring (32, 16, ..., 1) whose sweep shared memory fits in `limit`
-// bytes, or 0 if none does; and the sweep's own choice: with maps 80 KB a
+// bytes, or 0 if none does; and the sweep's own choice: with maps 108 KB a
 // CTA, two of which share an SM, else what one CTA may have.
 int sweep_ring_for(int sem_cap, int frame_depth, bool maps, size_t limit);
 int sweep_ring(int sem_cap, int frame_depth, bool maps);

@@ -86,7 +86,7 @@ struct sync_programs {
   int32_t* next_slot = nullptr;     // scratch: simulator's program-slot counter
   int32_t* fallback = nullptr;      // scratch: programs handed to the per-engine kernel
   int64_t max_inst = 0;             // instances of the largest program
-  int64_t n_stmt[2] = {0, 0};       // loop statements of all programs, of moving loops and fixed ones
+  syncgb::SweepCost sweep_cost{}, spec_cost{};   // barrier-free: of the programs, of the speculated pieces
   syncgb::BarArgs bar{};            // barrier scheme by intervals (bar.cuh)
   int32_t* todo = nullptr;          // scratch: programs the intervals leave to the sweep
   // program-order sweep
@@ -134,8 +134,7 @@ struct sync_programs {
   // none fits).  The maps' shared memory leaves room for up to 240 waited
   // semaphores, the walk's for 448: past the former the batch is walked.
   int sweep_choice(sync_sim_variant variant, int32_t sem_cap, int32_t frame_depth, bool& maps) const {
-    maps = variant != SYNC_SIM_BARRIER && syncgb::sweep_maps(sz.n_programs, sz.n_instances, n_stmt, num_sms) &&
-           syncgb::sweep_ring(sem_cap, frame_depth, true) > 0;
+    maps = variant != SYNC_SIM_BARRIER && syncgb::sweep_maps(sweep_cost, num_sms, sem_cap, frame_depth);
     return syncgb::sweep_ring(sem_cap, frame_depth, maps);
   }
 

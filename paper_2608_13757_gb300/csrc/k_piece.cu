@@ -335,10 +335,9 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
   if (L.n_spec > 0) {
     SweepArgs p = a;
     p.pcs.spec = 1;
-    // walked where no ring fits beside the maps (the caller's fits without)
-    p.ring = sweep_ring(p.sem_cap, p.frame_depth, true);
-    const bool maps = p.ring > 0;
-    if (!maps) p.ring = sweep_ring(p.sem_cap, p.frame_depth, false);
+    // (the caller's ring fits without the maps)
+    const bool maps = sweep_maps(L.spec_cost, num_sms, p.sem_cap, p.frame_depth);
+    p.ring = sweep_ring(p.sem_cap, p.frame_depth, maps);
     if (p.ring < 1) return cudaErrorInvalidConfiguration;
     const size_t smem = sweep_smem_bytes(p.sem_cap, p.frame_depth, p.ring, maps);
     p.pcs.probes = 1;

@@ -40,6 +40,36 @@ int sweep_ring(int sem_cap, int frame_depth, bool maps) {
   return r ? r : sweep_ring_for(sem_cap, frame_depth, maps, 200 * 1024);
 }
 
+// The maps' kernel runs 16 warps per SM, the walk's 24, or fewer where the
+// rings are large.  A sweep's time is taken as the longest item's and all
+// items' over the warps an SM runs at full rate (15.5, 10.7 or 6.9 walked with
+// 3, 2 or 1 CTAs, 8.8 or 6.3 by maps with 2 or 1), added as squares; the maps
+// have to promise 15%, what the estimate is off by.  Walked / by maps, us, one
+// loop of 16 records and trips of 64: 500 programs 557 / 209, 3000 829 / 564,
+// 20000 4240 / 2640; 4 records, trips of 32, 3000 236 / 359; 16 records, trips
+// of 8, 500 683 / 545, 3000 1027 / 1437; trips of 16, 3000 923 / 855, with 36
+// waited semaphores 923 / 1125, with 120 1954 / 1129; 40 records (no map),
+// 3000 15240 / 28570; two loops in turn (the warp keeps one map), 3000 6370 /
+// 9090; a loop entered once (never mapped), 3000 46 / 56; chain 777 9220 /
+// 6190, 4864 12600 / 9490; depth2 4096 4890 / 1150; sync-bound 65536 33960 /
+// 12510; branching trees 6000 844 / 1417.  Of many items the longest no longer
+// decide, and the estimate is good for loops of one size only: past 80 an SM
+// they need 320 instances a statement as well (chain 264, 16384 14.5 / 14.7
+// ms, 32768 16.4 / 21.3; depth2 540, 16384 7.0 / 4.3).
+bool sweep_maps(const SweepCost& c, int num_sms, int sem_cap, int frame_depth) {
+  const int ring_m = sweep_ring(sem_cap, frame_depth, true), ring_w = sweep_ring(sem_cap, frame_depth, false);
+  if (ring_m == 0) return false;
+  const auto ctas = [&](int ring, bool maps) {       // resident per SM, a kilobyte of which is the system's
+    return (int)(228 * 1024 / (sweep_smem_bytes(sem_cap, frame_depth, ring, maps) + 1024));
+  };
+  const int walked = ctas(ring_w, false), mapped = ctas(ring_m, true);
+  const double w = (double)c.walk / ((walked >= 3 ? 15.5 : walked == 2 ? 10.7 : 6.9) * num_sms);
+  const double m = (double)c.map / ((mapped >= 2 ? 8.8 : 6.3) * num_sms);
+  const double lw = (double)c.walk_max, lm = (double)c.map_max;
+  return lm * lm + m * m < 0.85 * 0.85 * (lw * lw + w * w) &&
+         (c.items <= 80 * num_sms || c.n_inst >= 320 * c.n_stmt[0] || c.n_stmt[1] >= 4 * c.n_stmt[0]);
+}
+
 cudaError_t launch_sweep(const SweepArgs& a, bool barrier, int num_sms, cudaStream_t s) {
   if (a.n_programs == 0) return cudaSuccess;
   if (a.ring < 1) return cudaErrorInvalidConfiguration;

@@ -150,6 +150,7 @@ struct alignas(16) ProgSummary {
   int64_t work;            // simulated work (the simulators' program order)
   int64_t n_inst;
   int64_t n_stmt[2];       // loop statements (on engine 0), of loops that are not fixed and of those that are
+  int64_t walk, map;       // a warp's cycles barrier-free: walked, and with trips by their maps (SweepCost)
   int64_t code_looped, code_unrolled;   // static instructions (code-size proxy)
   int64_t n_bar_deps;      // barrier-fallback dependencies
   int64_t struct_bytes;    // path entries and rowptr spaces the threshold kernels read
@@ -472,9 +473,25 @@ struct ProgBuilder {
     c[BC_PATH]++;
   }
 
+  // a loop that is not fixed, itself or around l
+  PB_HD int32_t host_of(int32_t l) const {
+    while (fixed(l)) l = par[l];
+    return l;
+  }
+  // a wait of an iteration of the consumer's host, for sweep_cost: its waits
+  // (33: none of a map) << 16 | those that are inputs of the map
+  PB_HD void count_wait(int32_t Cl, int32_t Sl, int32_t off) {
+    const int32_t h = host_of(Cl);
+    int32_t& w = S.cidx[l0 + h];
+    if (w >> 16 > 32) return;
+    if (Sl == h && off > 3) w = 33 << 16;          // farther than a map carries
+    else w += (1 << 16) + (off == 0 && host_of(Sl) == h ? 0 : 1);
+  }
+
   // dependencies: innermost common loop S, the cases of Sec. 5.2, N and K,
   // and everything the threshold kernels read for them
   PB_HD bool deps() {
+    for (int32_t l = 0; !FILL && l < nl; ++l) S.cidx[l0 + l] = 0;
     for (int64_t i = 0; i < (int64_t)nl * ne; ++i) {
       S.tstart[row0 + i] = -1;
       S.pe_of[row0 + i] = 0;
@@ -554,6 +571,7 @@ struct ProgBuilder {
         continue;
       }
       if (off > 0) S.needs_rhat[l0 + Sl] = 1;     // r-hat_S's no-wait check matters
+      if (!FILL) count_wait(Cl, Sl, off);
       const int32_t N = S.nloop_eng[row0 + (int64_t)Pl * ne + ep];
       const int32_t K = S.rank[x0 + px];
       if ((int64_t)N * tot(Pl, ep) > kI32Max) return fail(BE_N_OVERFLOW, k);
@@ -1136,6 +1154,76 @@ struct ProgBuilder {
       }
   }
 
+  // What one warp takes for the program barrier-free, in cycles of a warp with
+  // few neighbours: walked, and with trips by their maps where the sweep can
+  // build and use one (SweepCost in enc.h; trip.cuh has the conditions).
+  // Measured on one loop of 4 to 40 records, trips of 8 to 64: a loop
+  // statement 1400; a chunk of records 2000 with several iterations in it,
+  // 1500 with one, 2600 outside a leaf loop; a batch of up to 32 iterations
+  // by a map 1900 + 246 a record, and 34 + 5.2 a record for each iteration.
+  // (0.1 us a program, 1% of a chain batch's load.)
+  PB_HD void sweep_cost() {
+    constexpr int32_t kOut = 1 << 30;            // no map: a moving child loop or a fallback barrier
+    // COUNT's scratch from here on: the loops' costs at l * ne, and the loops
+    // that take the map's place, itself and below
+    int64_t* cost = S.tstart + row0;
+    const int32_t* waits = S.cidx + l0;
+    int32_t* cand = S.lfill + l0;
+    const int32_t* bp = bptr();
+    for (int32_t l = 0; l < nl; ++l) cand[l] = 0;
+    for (int32_t l = 1; l < nl; ++l) ++cand[par[l]];           // child loops
+    for (int32_t l = 0; l < nl; ++l) {
+      const int64_t t = tot(l, 0), np = n_parent(l, 0);
+      const int32_t nloops = cand[l], len = bp[l + 1] - bp[l] - nloops;
+      int64_t c = l > 0 ? np * 1400 : 0;
+      if (nloops > 0) c += len > 0 ? t * ((nloops < len ? nloops : len) + (len + 31) / 32) * 2600 : 0;
+      else if (len > 32) c += t * ((len + 31) / 32) * 2600;
+      else if (len > 16) c += t * 1500;
+      else if (len > 0) c += t * (2000 / (32 / len)) + np * 1000;
+      cost[(int64_t)l * ne] = c;
+      cand[l] = S.fbar[l0 + l] ? kOut : 0;
+    }
+    for (int32_t l = nl - 1; l > 0; --l) {       // children first
+      const int32_t q = par[l];
+      if (fixed(l)) {
+        cost[(int64_t)q * ne] += cost[(int64_t)l * ne];
+        cand[q] |= cand[l] & kOut;
+        continue;
+      }
+      if (!(cand[l] & kOut) && tot(l, 0) >= kTripMin * n_parent(l, 0) && tot(l, 0) > 0) ++cand[l];
+      else cand[l] |= kOut;
+      cand[q] = (cand[q] + (cand[l] & ~kOut)) | kOut;
+    }
+    sm.walk = cost[0];
+    double map = (double)cost[0];
+    for (int32_t l = 1; l < nl; ++l) {
+      if (fixed(l)) continue;
+      const int64_t c = cost[(int64_t)l * ne];
+      sm.walk += c;
+      map += (double)c;
+      if (cand[l] & kOut) continue;
+      const int32_t w = waits[l];
+      int32_t n_rec = 0, inputs = w & 0xffff;
+      for (int32_t e = 0; e < ne; ++e) {
+        n_rec += S.fix_cnt[row0 + (int64_t)l * ne + e];
+        inputs += S.fix_cnt[row0 + (int64_t)l * ne + e] > 0 ? 2 : 0;
+      }
+      if (n_rec < 1 || n_rec > 32 || w >> 16 > 32 || inputs > kTripCols) continue;
+      // the warp keeps one loop's map: a run of visits ends where another
+      // loop takes its place, and begins with kTripLearn walked iterations
+      int32_t a = l;
+      while (a != 0 && (cand[par[a]] & ~kOut) == 1) a = par[a];
+      const double visits = (double)n_parent(l, 0), runs = a == 0 ? 1 : (double)tot(par[a], 0);
+      const double trip = (double)tot(l, 0) / visits;
+      const double walked = (double)(int64_t)(trip >= kTripLearn ? 1 : (kTripLearn + trip - 1) / trip) * runs;
+      if (walked >= visits) continue;
+      const double batches = (double)(((int64_t)trip + 31) / 32);
+      const double one = batches * (1900 + 246 * n_rec) + trip * (34 + 5.2 * n_rec);
+      map += (visits - walked) * (one - ((double)c / visits - 1400));
+    }
+    sm.map = (int64_t)map;
+  }
+
   PB_HD void run() {
     bool ok = loops() && spaces() && instrs() && bodies();
     if (ok) {
@@ -1169,6 +1257,7 @@ struct ProgBuilder {
       sm.ne = ne;
       sm.n_inst = pi.n_inst;
       for (int32_t l = 1; l < nl; ++l) sm.n_stmt[fixed(l)] += tot(par[l], 0);
+      if (ok && !d.div) sweep_cost();
       sm.work = pi.n_inst + pi.n_pairs + (pi.n_stmt + pi.n_iter) * pi.ne;
       sm.splittable = !d.div && pi.fb_iters == 0;
       A.sum[p] = sm;

@@ -54,7 +54,6 @@ constexpr int SIM_FALLBACK = 9;             // internal: handed to the per-engin
 struct Frame { int32_t loop, item, g, g_end; };
 
 // A loop's trip map in shared memory, per warp (trip.cuh).
-constexpr int kTripCols = 24;               // inputs
 constexpr int kTripInts = 2 * 32 * kTripCols + 32 * (kTripCols + 1) + 64 + 7 * 32 + 8 * 32 + 16;
 
 // Shared memory of one warp (program), 16-byte aligned.

@@ -34,8 +34,6 @@ namespace syncgb {
 namespace {
 
 constexpr int32_t kTripNone = -(1 << 30);
-constexpr int kTripMin = 4;                 // shorter trips are walked
-constexpr int kTripLearn = 16;              // iterations walked before a loop's map is built
 constexpr int kTripRow = kTripCols + 1;     // odd: a lane per row without bank conflicts
 // the warp's ints (kTripInts)
 constexpr int kTripIn = 2 * 32 * kTripCols;         // [32][kTripRow] inputs per iteration
