@@ -39,7 +39,7 @@
  * instruction order; instruction x owns one int32 per global iteration of its
  * loop, starting at the sum of the instance counts of earlier instructions.
  *
- * Environment (read at each call; both only change how the work is split):
+ * Environment (read at each call; they only change how the work is split):
  *  - SYNCGB_LOAD_THREADS=n: host threads of sync_load_programs (default one
  *    per hardware thread, at most 32, at least 256 programs each).
  *  - SYNCGB_WIDE_INDEX=1: the threshold and check kernels index pairs with
@@ -48,6 +48,9 @@
  *    program needs to be simulated in pieces on several warps (default
  *    65536; see sync_simulate); SYNCGB_SPLIT_SPEC=1: such programs are
  *    always speculated, never probed, barrier-free.
+ *  - SYNCGB_INTERVAL_POOL=n: the most bytes of device memory that the
+ *    interval sums of a handle may take (default half of what is free; see
+ *    sync_simulate).
  */
 #ifndef SYNC_H
 #define SYNC_H
@@ -384,6 +387,11 @@ sync_status sync_check_minimal(const sync_programs *h, sync_thr_mode mode, const
  * The barrier scheme is evaluated by intervals between barriers, whose
  * schedules repeat, over all iterations at once; a program whose waits do not
  * repeat (checked on the thresholds of each call) is walked in program order.
+ * The first such call on a handle allocates the iterations' sums (device
+ * memory held by the handle: sync_sizes.device_bytes grows) and lays out the
+ * engines' positions in their streams, which depend on the batch alone; later
+ * calls reuse those and compute the times.  Where that memory is not to be
+ * had, every program is walked.
  * Barrier-free, large programs (sync_sizes.n_split_programs) whose top-level
  * body is one loop L are simulated in pieces -- runs of L's iterations -- on
  * separate warps when every wait of a piece targets an increment of the same

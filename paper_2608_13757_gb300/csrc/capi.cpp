@@ -727,9 +727,7 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   const size_t o_hist = L.add<int32_t>(hist_max), o_slot = L.add<int32_t>(kCounters + (int64_t)P);
   const size_t o_tile_first = L.add<int32_t>(n_first_tiles + 1), o_tile_job = L.add<int32_t>(n_job_tiles + 1);
   const int64_t n_tiles = cnt[BC_TILES];
-  // past this the interval starts would crowd out the batch itself: walked
-  const bool bar_fits = cnt[BC_FPOOL] <= kBarPoolMax;
-  const size_t o_tile_loop = L.add<int32_t>(n_tiles + 1), o_F = L.add<int32_t>(bar_fits ? cnt[BC_FPOOL] : 0);
+  const size_t o_tile_loop = L.add<int32_t>(n_tiles + 1);
   const size_t o_rel = L.add<int2>(n_ops), o_ko = L.add<int2>(NL), o_bind = L.add<uint8_t>(ND);
   const size_t o_left = L.add<int32_t>(P), o_counted = L.add<int32_t>(P), o_todo = L.add<int32_t>((int64_t)P + 1);
   char* dev = h.alloc<char>((int64_t)L.bytes, "encoding");
@@ -822,7 +820,8 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   h.next_slot = reinterpret_cast<int32_t*>(D(o_slot));
   h.fallback = h.next_slot + kCounters - 1;
   BarArgs& b = h.bar;
-  b.on = !div && bar_fits;
+  b.on = !div;
+  h.n_intervals = cnt[BC_FPOOL];
   b.n_tiles = (int32_t)n_tiles;
   b.bl = reinterpret_cast<BarLoop*>(D(o_bl));
   b.bdep = reinterpret_cast<BarDep*>(D(o_bdep));
@@ -837,7 +836,6 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   b.rel = reinterpret_cast<int2*>(D(o_rel));
   b.ko = reinterpret_cast<int2*>(D(o_ko));
   b.bind = reinterpret_cast<uint8_t*>(D(o_bind));
-  b.F = reinterpret_cast<int32_t*>(D(o_F));
   b.left = reinterpret_cast<int32_t*>(D(o_left));
   b.counted = reinterpret_cast<int32_t*>(D(o_counted));
   b.plans = h.next_slot + 1;
@@ -1114,6 +1112,30 @@ static int32_t* stored_times(const sync_programs* h, bool single) {
 
 // Both simulation entry points: thresholds from d_thr, or (fused) from the
 // simulators' loop state, optionally checked.
+// The interval pool of the barrier scheme (BarArgs::F), allocated on first
+// use; NULL, and the barrier scheme walked, where it does not fit: an
+// allocation that fails, or more than half of the device's free memory
+// (SYNCGB_INTERVAL_POOL=n: more than n bytes).  The next call asks again.
+static int32_t* interval_pool(const sync_programs* h) {
+  std::lock_guard<std::mutex> lock(h->intervals_mu);
+  if (h->intervals) return h->intervals;
+  const size_t bytes = (size_t)std::max<int64_t>(h->n_intervals, 1) * sizeof(int32_t);
+  if (const char* e = std::getenv("SYNCGB_INTERVAL_POOL")) {
+    if (bytes > (size_t)std::max(std::atoll(e), 0ll)) return nullptr;
+  } else if (bytes > ((size_t)64 << 20)) {      // (a smaller one is not worth the query)
+    size_t free_bytes = 0, total = 0;
+    cuda_check(cudaMemGetInfo(&free_bytes, &total), "cudaMemGetInfo");
+    if (bytes > free_bytes / 2) return nullptr;
+  }
+  void* p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    (void)cudaGetLastError();                   // not an error of the call
+    return nullptr;
+  }
+  const_cast<sync_programs*>(h)->own(p, bytes);
+  return h->intervals = static_cast<int32_t*>(p);
+}
+
 static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, const int32_t* d_thr,
                      const sync_sim_params* params,
                      sync_sim_variant variant, int32_t* d_makespan, unsigned long long* d_checksum,
@@ -1189,8 +1211,10 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
   const bool barrier = variant == SYNC_SIM_BARRIER;
   // barrier scheme: by intervals, in the sweep's launch or, with split
   // programs, in launches of its own
-  if (barrier && h->bar.on && h->max_inst >= kBarMinInst) {
+  int32_t* pool = barrier && h->bar.on && h->max_inst >= kBarMinInst ? interval_pool(h) : nullptr;
+  if (pool) {
     w.bar = h->bar;
+    w.bar.F = pool;
     if (const int r = sweep_ring_for(a.sem_cap, a.frame_depth, false, kBarRingBytes)) w.ring = r;
     w.bar.min_inst = kBarMinInst;
     if (h->n_split > 0) {
@@ -1239,6 +1263,8 @@ sync_status sync_simulate(const sync_programs* h, sync_thr_mode mode, const int3
     return SYNC_OK;
   } catch (const Failure& f) {
     return report(f);
+  } catch (const std::bad_alloc&) {
+    return report(Failure{SYNC_ERR_OOM, "host allocation failed"});
   }
 }
 
@@ -1252,6 +1278,8 @@ sync_status sync_simulate_fused(const sync_programs* h, sync_thr_mode mode, cons
     return SYNC_OK;
   } catch (const Failure& f) {
     return report(f);
+  } catch (const std::bad_alloc&) {
+    return report(Failure{SYNC_ERR_OOM, "host allocation failed"});
   }
 }
 

@@ -338,7 +338,7 @@ struct BarArgs {
   int2* ko;                  // scratch per loop: {duration of an iteration, offset in its parent's},
                              // both without the child loops' own durations
   uint8_t* bind;             // scratch per grouped dependency: 1 = waits inside its interval
-  int32_t* F;
+  int32_t* F;                // allocated on the handle's first barrier-scheme call
   int32_t* left;             // scratch per program: tiles left; kBarBad: a wait differs; < 0: not by intervals
   int32_t* counted;          // per program, zeroed at load: 1 = its counts (q >= 1) are in F
   int32_t* plans;            // zeroed per call: programs planned
@@ -350,7 +350,6 @@ constexpr int32_t kBarBad = 1 << 30;
 // by intervals).
 constexpr int32_t kBarMinInst = 256;
 constexpr size_t kBarRingBytes = 32 * 1024;
-constexpr int64_t kBarPoolMax = int64_t(8) << 30;   // entries of F: 32 GB
 // Counters a sweep launch starts from, zeroed together: next_slot[0], the
 // intervals' count of planned programs, fallback[0] (the list follows).
 constexpr int32_t kCounters = 3;

@@ -88,6 +88,9 @@ struct sync_programs {
   int64_t max_inst = 0;             // instances of the largest program
   syncgb::SweepCost sweep_cost{}, spec_cost{};   // barrier-free: of the programs, of the speculated pieces
   syncgb::BarArgs bar{};            // barrier scheme by intervals (bar.cuh)
+  int64_t n_intervals = 0;          // entries of its pool F
+  mutable std::mutex intervals_mu;
+  mutable int32_t* intervals = nullptr;   // F, allocated on first use
   int32_t* todo = nullptr;          // scratch: programs the intervals leave to the sweep
   // program-order sweep
   int32_t* plan_ptr = nullptr;
@@ -151,16 +154,25 @@ struct sync_programs {
     cudaSetDevice(prev);
   }
 
+  // memory the handle frees (lazily allocated tables of calls on several
+  // threads among it)
+  std::mutex blocks_mu;
+  void own(void* p, size_t bytes) {
+    std::lock_guard<std::mutex> lock(blocks_mu);
+    try {
+      blocks.push_back(p);
+    } catch (...) {
+      cudaFree(p);
+      throw;
+    }
+    sz.device_bytes += (int64_t)bytes;
+  }
   template <class V, class T = typename V::value_type>
   T* upload(const V& v, cudaStream_t s, const char* what) {
-    const size_t bytes = std::max<size_t>(v.size(), 1) * sizeof(T);
-    void* p = nullptr;
-    syncgb::cuda_or_raise(cudaMalloc(&p, bytes), what);
-    blocks.push_back(p);
-    sz.device_bytes += (int64_t)bytes;
+    T* p = alloc<T>((int64_t)v.size(), what);
     if (!v.empty()) syncgb::cuda_or_raise(cudaMemcpyAsync(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, s), what);
     sz.h2d_bytes += (int64_t)(v.size() * sizeof(T));
-    return static_cast<T*>(p);
+    return p;
   }
   // device memory the handle frees (mutable: lazily derived tables)
   template <class T>
@@ -172,8 +184,7 @@ struct sync_programs {
     const size_t bytes = (size_t)std::max<int64_t>(n, 1) * sizeof(T);
     void* p = nullptr;
     syncgb::cuda_or_raise(cudaMalloc(&p, bytes), what);
-    blocks.push_back(p);
-    sz.device_bytes += (int64_t)bytes;
+    own(p, bytes);
     return static_cast<T*>(p);
   }
 };

@@ -118,3 +118,57 @@ def test_thresholds_off_a_16_byte_boundary(sg, mode, at):
             assert torch.equal(getattr(got, f), getattr(want, f))
         assert not want.status.any()
     h.close()
+
+
+def device_bytes(sg, h):
+    import ctypes
+    s = sg.Sizes()
+    assert sg.lib().sync_query(h.handle, ctypes.byref(s)) == sg.OK
+    return s.device_bytes
+
+
+@pytest.mark.parametrize("split", [False, True], ids=["whole", "split"])
+def test_interval_pool_on_first_use(sg, split, monkeypatch):
+    """The iterations' sums take no memory from a handle that never simulates
+    the barrier scheme; a handle that may not have them walks, with the same
+    results; one that may takes them once."""
+    import torch
+    if split:
+        monkeypatch.setenv("SYNCGB_SPLIT_MIN", "1")
+    rng = np.random.default_rng(23)
+    batch = workloads.concat([program(total, 7, 9, 0.2, rng) for total in (1, 33, 129, 513)] +
+                             [workloads.generate("depth2", n_programs=3)])
+    # per loop around loops that do not run exactly once: starts and sums of the
+    # time and every engine's instances
+    entries = 0
+    for p in range(batch.n_programs):
+        l0, l1 = int(batch.prog_loop_ptr[p]), int(batch.prog_loop_ptr[p + 1])
+        trips = [batch.trips[batch.trip_ptr[l]:batch.trip_ptr[l + 1]] for l in range(l0, l1)]
+        par = batch.loop_parent[l0:l1]
+        once = [l > 0 and bool((trips[l] == 1).all()) for l in range(l1 - l0)]
+        for l in range(l1 - l0 - 1, 0, -1):
+            if not once[l]:
+                once[par[l]] = False
+        for l in range(l1 - l0):
+            if any(par[c] == l and not once[c] for c in range(l + 1, l1 - l0)):
+                entries += (1 + int(batch.prog_n_engines[p])) * (2 * int(trips[l].sum()) + 1)
+    h = sg.sync_load_programs(batch)
+    assert (h.sizes.n_split_programs > 0) == split
+    P, prm = batch.n_programs, sg.SimParams()
+    thr = sg.sync_eval_thresholds(h, oracle.PERLOOP)
+    sg.sync_simulate(h, oracle.PERLOOP, thr)             # barrier-free: the pieces' own scratch
+    loaded = device_bytes(sg, h)
+    ref = oracle.simulate(batch, oracle.thresholds(batch, oracle.PERLOOP), oracle.PERLOOP, oracle.BARRIER)
+    for limit, held in (("0", 0), (str(4 * entries - 1), 0), (str(4 * entries), 4 * entries), (None, 4 * entries),
+                        ("0", 4 * entries)):
+        if limit is None:
+            monkeypatch.delenv("SYNCGB_INTERVAL_POOL")
+        else:
+            monkeypatch.setenv("SYNCGB_INTERVAL_POOL", limit)
+        for r in (sg.sync_simulate(h, oracle.PERLOOP, thr, prm, oracle.BARRIER),
+                  sg.sync_simulate_fused(h, oracle.PERLOOP, prm, oracle.BARRIER)):
+            assert np.array_equal(r.status.cpu().numpy()[:P], ref.status)
+            assert np.array_equal(r.makespan.cpu().numpy()[:P], ref.makespan)
+            assert np.array_equal(r.checksum.cpu().numpy()[:P].view(np.uint64), ref.checksum)
+        assert device_bytes(sg, h) - loaded == held, limit
+    h.close()
