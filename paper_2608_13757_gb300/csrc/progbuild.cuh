@@ -479,13 +479,15 @@ struct ProgBuilder {
     return l;
   }
   // a wait of an iteration of the consumer's host, for sweep_cost: its waits
-  // (33: none of a map) << 16 | those that are inputs of the map
+  // (33: none of a map) << 16 | kNear if one reaches 1 or 2 iterations back |
+  // those that are inputs of the map
+  static constexpr int32_t kNear = 1 << 15;
   PB_HD void count_wait(int32_t Cl, int32_t Sl, int32_t off) {
     const int32_t h = host_of(Cl);
     int32_t& w = S.cidx[l0 + h];
     if (w >> 16 > 32) return;
     if (Sl == h && off > 3) w = 33 << 16;          // farther than a map carries
-    else w += (1 << 16) + (off == 0 && host_of(Sl) == h ? 0 : 1);
+    else w = (w + (1 << 16) + (off == 0 && host_of(Sl) == h ? 0 : 1)) | (Sl == h && off - 1u < 2u ? kNear : 0);
   }
 
   // dependencies: innermost common loop S, the cases of Sec. 5.2, N and K,
@@ -1158,10 +1160,11 @@ struct ProgBuilder {
   // few neighbours: walked, and with trips by their maps where the sweep can
   // build and use one (SweepCost in enc.h; trip.cuh has the conditions).
   // Measured on one loop of 4 to 40 records, trips of 8 to 64: a loop
-  // statement 1400; a chunk of records 2000 with several iterations in it,
-  // 1500 with one, 2600 outside a leaf loop; a batch of up to 32 iterations
-  // by a map 1900 + 246 a record, and 34 + 5.2 a record for each iteration.
-  // (0.1 us a program, 1% of a chain batch's load.)
+  // statement 1400; a chunk of records 2300 with 2 or 3 iterations in it, 2000
+  // with 4 or 5, 1500 with more and with one, each 1300 without waits inside
+  // it, 2600 outside a leaf loop; a batch of up to 32 iterations by a map 1900
+  // + 246 a record, and 34 + 5.2 a record for each iteration; building the
+  // map 2000 an input.  (0.1 us a program, 1% of a chain batch's load.)
   PB_HD void sweep_cost() {
     constexpr int32_t kOut = 1 << 30;            // no map: a moving child loop or a fallback barrier
     // COUNT's scratch from here on: the loops' costs at l * ne, and the loops
@@ -1176,10 +1179,13 @@ struct ProgBuilder {
       const int64_t t = tot(l, 0), np = n_parent(l, 0);
       const int32_t nloops = cand[l], len = bp[l + 1] - bp[l] - nloops;
       int64_t c = l > 0 ? np * 1400 : 0;
+      // waits inside a chunk take more passes over it
+      const int32_t w = waits[l];
+      const bool inner = w >> 16 > (w & (kNear - 1)) || (len <= 10 && (w & kNear));
       if (nloops > 0) c += len > 0 ? t * ((nloops < len ? nloops : len) + (len + 31) / 32) * 2600 : 0;
       else if (len > 32) c += t * ((len + 31) / 32) * 2600;
-      else if (len > 16) c += t * 1500;
-      else if (len > 0) c += t * (2000 / (32 / len)) + np * 1000;
+      else if (len > 16) c += t * (inner ? 1500 : 1300);
+      else if (len > 0) c += t * ((!inner ? 1300 : len > 8 ? 2300 : len > 5 ? 2000 : 1500) / (32 / len)) + np * 1000;
       cost[(int64_t)l * ne] = c;
       cand[l] = S.fbar[l0 + l] ? kOut : 0;
     }
@@ -1203,7 +1209,7 @@ struct ProgBuilder {
       map += (double)c;
       if (cand[l] & kOut) continue;
       const int32_t w = waits[l];
-      int32_t n_rec = 0, inputs = w & 0xffff;
+      int32_t n_rec = 0, inputs = w & (kNear - 1);
       for (int32_t e = 0; e < ne; ++e) {
         n_rec += S.fix_cnt[row0 + (int64_t)l * ne + e];
         inputs += S.fix_cnt[row0 + (int64_t)l * ne + e] > 0 ? 2 : 0;
@@ -1219,7 +1225,7 @@ struct ProgBuilder {
       if (walked >= visits) continue;
       const double batches = (double)(((int64_t)trip + 31) / 32);
       const double one = batches * (1900 + 246 * n_rec) + trip * (34 + 5.2 * n_rec);
-      map += (visits - walked) * (one - ((double)c / visits - 1400));
+      map += runs * 2000 * inputs + (visits - walked) * (one - ((double)c / visits - 1400));
     }
     sm.map = (int64_t)map;
   }

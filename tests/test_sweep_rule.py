@@ -82,6 +82,27 @@ def test_configurations(config, programs, maps):
     assert takes_maps(workloads.generate(config, n_programs=programs)) == maps
 
 
+def test_waits_inside_a_chunk_make_the_walk_longer():
+    """A body without waits inside an iteration is walked in one pass a chunk:
+    the same loop in many programs stays with the walk."""
+    b = workloads.ProgramBuilder(5)
+    A = b.loop(0, 0, [18])
+    L = b.loop(A, 0, [6, 7, 7, 8, 9, 11, 13, 18, 18, 21, 24, 25, 26, 27, 28, 30, 31, 32])
+    xs = [b.instr(L, i, i % 5, 10 + i) for i in range(12)]
+    for i in range(3):
+        b.dep(xs[i], xs[i + 4], 2)
+    apart = b.batch()
+    for i in range(1, 12, 2):
+        b.dep(xs[i - 1], xs[i], 0)
+    assert takes_maps(apart) and not takes_maps(many(apart, 3000))
+    assert takes_maps(b.batch()) and takes_maps(many(b.batch(), 3000))
+
+
+@pytest.mark.parametrize("shape", [(8, 16, 4, 1), (4, 16, 16, 1), (4, 64, 4, 1)])
+def test_building_the_map_has_to_pay(shape):
+    assert not takes_maps(leaves(*shape)) and not takes_maps(many(leaves(*shape), 1000))
+
+
 def test_waited_semaphores():
     """Rings that leave the maps one CTA per SM and the walk three, two and
     one, and no ring beside the maps."""
