@@ -388,7 +388,8 @@ sync_status sync_check_minimal(const sync_programs *h, sync_thr_mode mode, const
  * schedules repeat, over all iterations at once; a program whose waits do not
  * repeat (checked on the thresholds of each call) is walked in program order.
  * The first such call on a handle allocates the iterations' sums (device
- * memory held by the handle: sync_sizes.device_bytes grows) and lays out the
+ * memory held by the handle: sync_sizes.device_bytes grows; up to 16 MB come
+ * with the encoding) and lays out the
  * engines' positions in their streams, which depend on the batch alone; later
  * calls reuse those and compute the times.  Where that memory is not to be
  * had, every program is walked.

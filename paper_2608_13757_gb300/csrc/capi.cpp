@@ -237,6 +237,13 @@ static int64_t split_floor() {
   return min_inst;
 }
 
+// The most bytes a handle's interval pool may take (SYNCGB_INTERVAL_POOL=n).
+static int64_t interval_limit() {
+  const char* e = std::getenv("SYNCGB_INTERVAL_POOL");
+  return e ? std::max(std::atoll(e), 0ll) : INT64_MAX;
+}
+constexpr int64_t kIntervalsInBlock = 16 << 20;
+
 // Piece-parallel simulation (PieceArgs in enc.h): which programs are split,
 // into which pieces, and what each piece starts from.  A program qualifies
 // when its top-level body is one loop L (no instruction of its own), its
@@ -728,6 +735,10 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   const size_t o_tile_first = L.add<int32_t>(n_first_tiles + 1), o_tile_job = L.add<int32_t>(n_job_tiles + 1);
   const int64_t n_tiles = cnt[BC_TILES];
   const size_t o_tile_loop = L.add<int32_t>(n_tiles + 1);
+  // a small interval pool comes with the encoding: an allocation of its own
+  // takes about 0.1 ms of the first call
+  const bool pool_here = cnt[BC_FPOOL] * (int64_t)sizeof(int32_t) <= std::min(interval_limit(), kIntervalsInBlock);
+  const size_t o_F = L.add<int32_t>(pool_here ? cnt[BC_FPOOL] : 0);
   const size_t o_rel = L.add<int2>(n_ops), o_ko = L.add<int2>(NL), o_bind = L.add<uint8_t>(ND);
   const size_t o_left = L.add<int32_t>(P), o_counted = L.add<int32_t>(P), o_todo = L.add<int32_t>((int64_t)P + 1);
   char* dev = h.alloc<char>((int64_t)L.bytes, "encoding");
@@ -822,6 +833,7 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   BarArgs& b = h.bar;
   b.on = !div;
   h.n_intervals = cnt[BC_FPOOL];
+  if (pool_here) h.intervals = reinterpret_cast<int32_t*>(D(o_F));
   b.n_tiles = (int32_t)n_tiles;
   b.bl = reinterpret_cast<BarLoop*>(D(o_bl));
   b.bdep = reinterpret_cast<BarDep*>(D(o_bdep));
@@ -1119,20 +1131,19 @@ static int32_t* stored_times(const sync_programs* h, bool single) {
 static int32_t* interval_pool(const sync_programs* h) {
   std::lock_guard<std::mutex> lock(h->intervals_mu);
   if (h->intervals) return h->intervals;
-  const size_t bytes = (size_t)std::max<int64_t>(h->n_intervals, 1) * sizeof(int32_t);
-  if (const char* e = std::getenv("SYNCGB_INTERVAL_POOL")) {
-    if (bytes > (size_t)std::max(std::atoll(e), 0ll)) return nullptr;
-  } else if (bytes > ((size_t)64 << 20)) {      // (a smaller one is not worth the query)
+  const int64_t bytes = h->n_intervals * (int64_t)sizeof(int32_t);
+  if (bytes > interval_limit()) return nullptr;
+  if (!std::getenv("SYNCGB_INTERVAL_POOL")) {
     size_t free_bytes = 0, total = 0;
     cuda_check(cudaMemGetInfo(&free_bytes, &total), "cudaMemGetInfo");
-    if (bytes > free_bytes / 2) return nullptr;
+    if ((size_t)bytes > free_bytes / 2) return nullptr;
   }
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+  if (cudaMalloc(&p, (size_t)bytes) != cudaSuccess) {
     (void)cudaGetLastError();                   // not an error of the call
     return nullptr;
   }
-  const_cast<sync_programs*>(h)->own(p, bytes);
+  const_cast<sync_programs*>(h)->own(p, (size_t)bytes);
   return h->intervals = static_cast<int32_t*>(p);
 }
 

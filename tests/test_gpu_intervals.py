@@ -129,10 +129,10 @@ def device_bytes(sg, h):
 
 @pytest.mark.parametrize("split", [False, True], ids=["whole", "split"])
 def test_interval_pool_on_first_use(sg, split, monkeypatch):
-    """The iterations' sums take no memory from a handle that never simulates
-    the barrier scheme; a handle that may not have them walks, with the same
-    results; one that may takes them once."""
-    import torch
+    """The iterations' sums are allocated on the first barrier-scheme call
+    (unless they are small enough to come with the encoding); a handle that
+    may not have them walks, with the same results; one that may takes them
+    once."""
     if split:
         monkeypatch.setenv("SYNCGB_SPLIT_MIN", "1")
     rng = np.random.default_rng(23)
@@ -153,6 +153,11 @@ def test_interval_pool_on_first_use(sg, split, monkeypatch):
             if any(par[c] == l and not once[c] for c in range(l + 1, l1 - l0)):
                 entries += (1 + int(batch.prog_n_engines[p])) * (2 * int(trips[l].sum()) + 1)
     h = sg.sync_load_programs(batch)
+    with_pool = h.sizes.device_bytes
+    h.close()
+    monkeypatch.setenv("SYNCGB_INTERVAL_POOL", "0")
+    h = sg.sync_load_programs(batch)
+    assert abs(with_pool - h.sizes.device_bytes - 4 * entries) < 512      # (alignment)
     assert (h.sizes.n_split_programs > 0) == split
     P, prm = batch.n_programs, sg.SimParams()
     thr = sg.sync_eval_thresholds(h, oracle.PERLOOP)
