@@ -48,6 +48,9 @@
  *    program needs to be simulated in pieces on several warps (default
  *    65536; see sync_simulate); SYNCGB_SPLIT_SPEC=1: such programs are
  *    always speculated, never probed, barrier-free.
+ *  - SYNCGB_INTERVALS=1 or 0 (read by sync_load_programs): the barrier scheme
+ *    takes every program, or none, by intervals (default: those whose walk is
+ *    estimated longer; see sync_simulate).
  *  - SYNCGB_INTERVAL_POOL=n: the most bytes of device memory that the
  *    interval sums of a handle may take (default half of what is free; see
  *    sync_simulate).
@@ -386,7 +389,8 @@ sync_status sync_check_minimal(const sync_programs *h, sync_thr_mode mode, const
  * update and c_regop per pair of a wait with a cached-sum read.
  * The barrier scheme is evaluated by intervals between barriers, whose
  * schedules repeat, over all iterations at once; a program whose waits do not
- * repeat (checked on the thresholds of each call) is walked in program order.
+ * repeat (checked on the thresholds of each call), or whose walk is estimated
+ * shorter than laying out its intervals, is walked in program order.
  * The first such call on a handle allocates the iterations' sums (device
  * memory held by the handle: sync_sizes.device_bytes grows; up to 16 MB come
  * with the encoding) and lays out the

@@ -411,7 +411,7 @@ template <int MODE, bool FUSED>
 __device__ __noinline__ bool bar_plan(const SweepArgs& a, int p, int32_t* at, int lane) {
   const ProgInfo pi = a.prog[p];
   const BarProg b = bar_prog(pi);
-  bool ok = pi.n_inst >= a.bar.min_inst && bar_in_time<MODE>(a, pi);
+  bool ok = (pi.intervals & a.bar.which) && bar_in_time<MODE>(a, pi);
   if (ok) {
     bar_counts(a, p, pi, lane);
     ok = bar_classes<MODE, FUSED>(a, pi, lane);

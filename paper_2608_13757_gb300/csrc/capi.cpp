@@ -743,6 +743,9 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
   const size_t o_left = L.add<int32_t>(P), o_counted = L.add<int32_t>(P), o_todo = L.add<int32_t>((int64_t)P + 1);
   char* dev = h.alloc<char>((int64_t)L.bytes, "encoding");
 
+  if (const char* e = std::getenv("SYNCGB_INTERVALS"))       // every program, or none, by intervals (tests)
+    for (int32_t p = 0; p < P; ++p) a.sum[p].intervals = e[0] == '1' && !div ? 15 : 0;
+
   // ------------------------------------------------------------- FILL
   ArenaLease AL(host_bytes, device);
   char* host = AL.a->p;
@@ -865,7 +868,7 @@ static void build(const sync_batch_desc& d, int device, cudaStream_t stream, syn
     code_looped += s.code_looped;
     code_unrolled += s.code_unrolled;
     n_bar_deps += s.n_bar_deps;
-    h.max_inst = std::max(h.max_inst, s.n_inst);
+    h.by_intervals |= s.intervals;
     add_cost(h.sweep_cost, s, 1);
     ne_max = std::max(ne_max, s.ne);
     depth_max = std::max(depth_max, s.depth_max);
@@ -933,6 +936,23 @@ static void validate(const sync_batch_desc& d) {
   int64_t tot[kBuildCounts];
   Team team(load_threads(sh.covered));
   count_pass(d, sh, team, *SL.s, a, tot);
+}
+
+// For the tests of the dispatch (not part of the interface, no CUDA call):
+// ProgInfo::intervals of the batch's first program, -1 for a batch that does
+// not load.
+extern "C" int syncgb_by_intervals(const sync_batch_desc* desc) {
+  try {
+    const Shape sh = shape_checks(*desc);
+    ScratchLease SL;
+    BuildArgs a{};
+    int64_t tot[kBuildCounts];
+    Team team(load_threads(sh.covered));
+    count_pass(*desc, sh, team, *SL.s, a, tot);
+    return sh.P > 0 ? a.sum[0].intervals : 0;
+  } catch (...) {
+    return -1;
+  }
 }
 
 // For the tests of the dispatch (not part of the interface, no CUDA call):
@@ -1222,12 +1242,13 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
   const bool barrier = variant == SYNC_SIM_BARRIER;
   // barrier scheme: by intervals, in the sweep's launch or, with split
   // programs, in launches of its own
-  int32_t* pool = barrier && h->bar.on && h->max_inst >= kBarMinInst ? interval_pool(h) : nullptr;
+  const int32_t which = h->sz.n_programs <= kBarFew * h->num_sms ? 1 : 2;
+  int32_t* pool = barrier && h->bar.on && (h->by_intervals & which) ? interval_pool(h) : nullptr;
   if (pool) {
     w.bar = h->bar;
     w.bar.F = pool;
     if (const int r = sweep_ring_for(a.sem_cap, a.frame_depth, false, kBarRingBytes)) w.ring = r;
-    w.bar.min_inst = kBarMinInst;
+    w.bar.which = which << 2;
     if (h->n_split > 0) {
       cuda_check(launch_intervals(w, h->todo, h->sz.n_loops, st), "interval simulation");
       w.bar.on = 0;

@@ -83,7 +83,8 @@ struct alignas(16) ProgInfo {
   int32_t divergent;  // 1: engines run their own trip counts (per-engine kernel only)
   int32_t nloops;
   int32_t dep0, ndep; // its consumer-grouped dependencies [dep0, dep0 + ndep)
-  int32_t pad_;
+  int32_t intervals;  // barrier scheme by intervals, in a batch of few programs (bits 0 and 2) or of many
+                      // (1 and 3): worth a batch's while, and worth it beside such a program
 };
 
 // Program-order sweep tables.  Per loop, a plan: its body cut at child loops
@@ -322,7 +323,7 @@ struct alignas(16) BarDep {
 struct BarArgs {
   int32_t on;                // 1: the sweep launch runs the intervals first (bar.cuh)
   int32_t n_tiles;
-  int32_t min_inst;          // programs with fewer instances are swept
+  int32_t which;             // the bit of ProgInfo::intervals that sends a program here; the others are swept
   const BarLoop* bl;
   const BarDep* bdep;
   const int2* rowc;          // per (loop, engine): instances {before it in its parent's (fixed: its host's)
@@ -345,10 +346,20 @@ struct BarArgs {
   const int32_t* todo;       // sweep only these: [0] count, [1..] programs (NULL: all)
 };
 constexpr int32_t kBarBad = 1 << 30;
-// Programs with fewer instances are swept: a plan is a chain of about 30 us,
-// what the walk takes for 300 instances (one program of 96: 18 us swept, 36
-// by intervals).
-constexpr int32_t kBarMinInst = 256;
+// A batch goes by intervals where the walk of one of its programs is estimated
+// longer than its plan (sweep_cost in progbuild.cuh); a program of it is still
+// walked, in that launch, where its walk is shorter than half its plan (the
+// launch's walk has fewer registers, and holds up the warp's tiles: depth2
+// 4096 with the small programs walked 428 us, by intervals 356).  Few
+// programs, at most kBarFew an SM, wait for one plan's chain of dependent
+// steps; many for the plans' instructions, most of them the segments'.  Walked
+// / by intervals, us: a loop of 16 records and trips of 64, entered once 43 /
+// 67 for one program, 54 / 75 for 3000, 115 / 206 for 12000; 4 times 92 / 68,
+// 127 / 137 and 377 / 237; 16 times 282 / 69 and 423 / 192; a small nest of a
+// chain program (262 instances, 3 segments) 32 / 56 and 40 / 104, a larger one
+// (2054, 5 segments) 136 / 78 and 194 / 149; a branching tree (722, 11
+// segments) 121 / 110 and 174 / 244.
+constexpr int kBarFew = 8;
 constexpr size_t kBarRingBytes = 32 * 1024;
 // Counters a sweep launch starts from, zeroed together: next_slot[0], the
 // intervals' count of planned programs, fallback[0] (the list follows).

@@ -85,7 +85,7 @@ struct sync_programs {
   int32_t* hist = nullptr;          // scratch: retire time of each semaphore increment
   int32_t* next_slot = nullptr;     // scratch: simulator's program-slot counter
   int32_t* fallback = nullptr;      // scratch: programs handed to the per-engine kernel
-  int64_t max_inst = 0;             // instances of the largest program
+  int32_t by_intervals = 0;         // ProgInfo::intervals of all programs, or'ed
   syncgb::SweepCost sweep_cost{}, spec_cost{};   // barrier-free: of the programs, of the speculated pieces
   syncgb::BarArgs bar{};            // barrier scheme by intervals (bar.cuh)
   int64_t n_intervals = 0;          // entries of its pool F

@@ -151,6 +151,7 @@ struct alignas(16) ProgSummary {
   int64_t n_inst;
   int64_t n_stmt[2];       // loop statements (on engine 0), of loops that are not fixed and of those that are
   int64_t walk, map;       // a warp's cycles barrier-free: walked, and with trips by their maps (SweepCost)
+  int32_t intervals;       // ProgInfo::intervals
   int64_t code_looped, code_unrolled;   // static instructions (code-size proxy)
   int64_t n_bar_deps;      // barrier-fallback dependencies
   int64_t struct_bytes;    // path entries and rowptr spaces the threshold kernels read
@@ -480,13 +481,14 @@ struct ProgBuilder {
   }
   // a wait of an iteration of the consumer's host, for sweep_cost: its waits
   // (33: none of a map) << 16 | kNear if one reaches 1 or 2 iterations back |
+  // kMany if an instruction has more than the sweep holds in registers |
   // those that are inputs of the map
-  static constexpr int32_t kNear = 1 << 15;
+  static constexpr int32_t kNear = 1 << 15, kMany = 1 << 14;
   PB_HD void count_wait(int32_t Cl, int32_t Sl, int32_t off) {
     const int32_t h = host_of(Cl);
     int32_t& w = S.cidx[l0 + h];
     if (w >> 16 > 32) return;
-    if (Sl == h && off > 3) w = 33 << 16;          // farther than a map carries
+    if (Sl == h && off > 3) w = 33 << 16 | (w & kNear);          // farther than a map carries
     else w = (w + (1 << 16) + (off == 0 && host_of(Sl) == h ? 0 : 1)) | (Sl == h && off - 1u < 2u ? kNear : 0);
   }
 
@@ -700,7 +702,7 @@ struct ProgBuilder {
       const int32_t cx = d.dep_cons[gd], lev = levels(d.dep_prod[gd]);
       S.x_levels[x0 + cx] += lev;
       pi.pair_levels += (int64_t)lev * tot(IL(cx), IE(cx));
-      S.x_ndeps[x0 + cx]++;
+      if (++S.x_ndeps[x0 + cx] > 2) S.cidx[l0 + IL(cx)] |= kMany;
     }
     for (int32_t x = 0, at = 0; x < nx; ++x) {
       if (S.x_ndeps[x0 + x] > 0) S.x_dep_begin[x0 + x] = d0 + at;
@@ -1173,17 +1175,35 @@ struct ProgBuilder {
     const int32_t* waits = S.cidx + l0;
     int32_t* cand = S.lfill + l0;
     const int32_t* bp = bptr();
+    // the barrier scheme's walk: a visit 3000 and an iteration of a leaf loop
+    // 500, which replays the schedule of the one before it (the first ones of
+    // a trip 1500 more), 2700 where a record has more waits than registers; a
+    // chunk elsewhere 1500 or 2700; a conditional around one record 1700
+    int64_t barrier = 0, segs = 0, recs = 0, loops = 0, sibs = 0;
     for (int32_t l = 0; l < nl; ++l) cand[l] = 0;
     for (int32_t l = 1; l < nl; ++l) ++cand[par[l]];           // child loops
     for (int32_t l = 0; l < nl; ++l) {
       const int64_t t = tot(l, 0), np = n_parent(l, 0);
       const int32_t nloops = cand[l], len = bp[l + 1] - bp[l] - nloops;
+      const int32_t cuts = nloops < len ? nloops : len, chunks = (len + 31) / 32;
+      const int64_t live = np < t ? np : t, far = live * (waits[l] & kNear ? 3 : 1);
+      if (l > 0) barrier += np * 1400;
+      if (nloops > 0) barrier += live * 1600 + t * ((len > 0 ? cuts + chunks : 0) * 1500 + 400);
+      else if (len == 1 && t <= np) barrier += t * 300;
+      else if (len > 32 || (waits[l] & kMany)) barrier += live * 1600 + t * chunks * 2700;
+      else if (len > 0) barrier += live * 1600 + t * 500 + (far < t ? far : t) * 1500;
+      if (t > 0) {
+        segs += len == 0 ? 0 : nloops == 0 ? 1 : nloops < len ? nloops + 1 : len;
+        ++loops;
+        sibs += nloops > 1 ? nloops - 1 : 0;
+      }
+      recs += len;
       int64_t c = l > 0 ? np * 1400 : 0;
       // waits inside a chunk take more passes over it
       const int32_t w = waits[l];
-      const bool inner = w >> 16 > (w & (kNear - 1)) || (len <= 10 && (w & kNear));
-      if (nloops > 0) c += len > 0 ? t * ((nloops < len ? nloops : len) + (len + 31) / 32) * 2600 : 0;
-      else if (len > 32) c += t * ((len + 31) / 32) * 2600;
+      const bool inner = w >> 16 > (w & (kMany - 1)) || (len <= 10 && (w & kNear));
+      if (nloops > 0) c += len > 0 ? t * (cuts + chunks) * 2600 : 0;
+      else if (len > 32) c += t * chunks * 2600;
       else if (len > 16) c += t * (inner ? 1500 : 1300);
       else if (len > 0) c += t * ((!inner ? 1300 : len > 8 ? 2300 : len > 5 ? 2000 : 1500) / (32 / len)) + np * 1000;
       cost[(int64_t)l * ne] = c;
@@ -1200,6 +1220,12 @@ struct ProgBuilder {
       else cand[l] |= kOut;
       cand[q] = (cand[q] + (cand[l] & ~kOut)) | kOut;
     }
+    // laying out its intervals: for few programs the chain of steps, for many
+    // all their work (siblings' tiles look up each other's sums)
+    const int64_t few = 19000 + 7500 * (segs + loops) + 9000 * sibs + 1500 * recs;
+    const int64_t all = 19000 * segs + 6400 * loops + 45000 * sibs + 1000 * recs + 7 * pi.n_inst;
+    sm.intervals = (barrier > few ? 1 : 0) | (barrier > all ? 2 : 0) | (2 * barrier > few ? 4 : 0) |
+                   (2 * barrier > all ? 8 : 0);
     sm.walk = cost[0];
     double map = (double)cost[0];
     for (int32_t l = 1; l < nl; ++l) {
@@ -1209,7 +1235,7 @@ struct ProgBuilder {
       map += (double)c;
       if (cand[l] & kOut) continue;
       const int32_t w = waits[l];
-      int32_t n_rec = 0, inputs = w & (kNear - 1);
+      int32_t n_rec = 0, inputs = w & (kMany - 1);
       for (int32_t e = 0; e < ne; ++e) {
         n_rec += S.fix_cnt[row0 + (int64_t)l * ne + e];
         inputs += S.fix_cnt[row0 + (int64_t)l * ne + e] > 0 ? 2 : 0;
@@ -1251,6 +1277,7 @@ struct ProgBuilder {
       reads();
     }
     if constexpr (FILL) {
+      pi.intervals = A.sum[p].intervals;
       O.prog[p] = pi;
       if (p == d.P - 1) {                        // the closing entries of the offset tables
         O.seg[d.ND] = c[BC_PADDED];

@@ -26,6 +26,12 @@ def sg():
     return m
 
 
+@pytest.fixture(autouse=True)
+def every_program_by_intervals(monkeypatch):
+    """The shapes here are small: by default most would be walked."""
+    monkeypatch.setenv("SYNCGB_INTERVALS", "1")
+
+
 def trips_of(total, rows, empty, rng):
     """`rows` trips that add up to `total`, a share `empty` of them 0."""
     t = np.zeros(rows, dtype=np.int64)
@@ -177,3 +183,18 @@ def test_interval_pool_on_first_use(sg, split, monkeypatch):
             assert np.array_equal(r.checksum.cpu().numpy()[:P].view(np.uint64), ref.checksum)
         assert device_bytes(sg, h) - loaded == held, limit
     h.close()
+
+
+@pytest.mark.parametrize("programs", [3, 1217])
+@pytest.mark.parametrize("by", ["0", "1", None], ids=["walk", "intervals", "estimate"])
+def test_walked_beside_planned(sg, by, programs, monkeypatch):
+    """Programs on both sides of the estimate in one batch, few and many
+    (more than 8 an SM), and each scheme for all of them."""
+    if by is None:
+        monkeypatch.delenv("SYNCGB_INTERVALS")
+    else:
+        monkeypatch.setenv("SYNCGB_INTERVALS", by)
+    rng = np.random.default_rng(31)
+    some = workloads.concat([program(total, 7, 9, 0.2, rng) for total in (1, 40, 400)])
+    batch = workloads.concat([some] * (programs // 3) + [workloads.generate("depth2", n_programs=2)])
+    compare_all(sg, batch, modes=[oracle.PERLOOP])

@@ -1,7 +1,9 @@
 """Which barrier-free batches take trips by their maps (sweep_maps in
-csrc/enc.h), on the host: only those whose loops a map can take for most of
-their work -- trips that follow each other, of bodies up to 32 records, after
-the iterations walked first -- and whose gain outweighs the fewer warps."""
+csrc/k_sweep.cu), on the host: only those whose loops a map can take for most
+of their work -- trips that follow each other, of bodies up to 32 records,
+after the iterations walked first -- and whose gain outweighs the fewer warps.
+And which programs the barrier scheme takes by intervals: those whose walk is
+longer than laying them out."""
 import ctypes
 
 import numpy as np
@@ -145,3 +147,18 @@ def test_refused_batch():
     b.instr_latency[:] = 0
     desc, keep = sg.batch_desc(b)
     assert sg.lib().syncgb_takes_maps(ctypes.byref(desc), SMS, 4) == -1 and keep
+
+
+@pytest.mark.parametrize("shape,few,many_", [
+    ((16, 64, 1, 1), False, False),       # one trip: its iterations replay
+    ((24, 16, 4, 1), False, False),
+    ((8, 16, 2, 2), False, False),        # sibling loops
+    ((16, 64, 16, 1), True, True),
+    ((2, 4, 32, 1), True, True),          # short trips
+    ((40, 32, 4, 1), True, True),         # more records than lanes
+    ((5, 16, 8, 1, 5), True, True)])      # conditionals around one record
+def test_programs_by_intervals(shape, few, many_):
+    desc, keep = sg.batch_desc(leaves(*shape))
+    got = sg.lib().syncgb_by_intervals(ctypes.byref(desc))
+    assert keep and (got & 1, got & 2) == (1 if few else 0, 2 if many_ else 0)
+    assert not got & 3 or got >> 2 & got & 3 == got & 3
