@@ -44,10 +44,10 @@ int sweep_ring(int sem_cap, int frame_depth, bool maps) {
 // rings are large.  A sweep's time is taken as the longest item's and all
 // items' over the warps an SM runs at full rate (15.5, 10.7 or 6.9 walked with
 // 3, 2 or 1 CTAs, 8.8 or 6.3 by maps with 2 or 1), added as squares; the maps
-// have to promise 15%, what the estimate is off by, or 5% where the longest
-// item makes the time.  Walked / by maps, us, one
-// loop of 16 records and trips of 64: 500 programs 557 / 209, 3000 829 / 564,
-// 20000 4240 / 2640; 4 records, trips of 32, 3000 236 / 359; 16 records, trips
+// have to promise 9%, or 5% where the longest item makes the time.  Walked / by
+// maps, us, one loop of 16 records and trips of 64: 500 programs 557 / 209,
+// 3000 829 / 564, 20000 4240 / 2640; 12 records without waits inside an
+// iteration, trips of 19, 3000 296 / 424; 4 records, trips of 32, 3000 236 / 359; 16 records, trips
 // of 8, 500 683 / 545, 3000 1027 / 1437; trips of 16, 3000 923 / 855, with 36
 // waited semaphores 923 / 1125, with 120 1954 / 1129; 40 records (no map),
 // 3000 15240 / 28570; two loops in turn (the warp keeps one map), 3000 6370 /
@@ -67,7 +67,7 @@ bool sweep_maps(const SweepCost& c, int num_sms, int sem_cap, int frame_depth) {
   const double w = (double)c.walk / ((walked >= 3 ? 15.5 : walked == 2 ? 10.7 : 6.9) * num_sms);
   const double m = (double)c.map / ((mapped >= 2 ? 8.8 : 6.3) * num_sms);
   const double lw = (double)c.walk_max, lm = (double)c.map_max;
-  const double most = m < lm / 2 ? 0.95 : 0.85;
+  const double most = m < lm / 2 ? 0.95 : 0.91;
   return lm * lm + m * m < most * most * (lw * lw + w * w) &&
          (c.items <= 80 * num_sms || c.n_inst >= 320 * c.n_stmt[0] || c.n_stmt[1] >= 4 * c.n_stmt[0]);
 }

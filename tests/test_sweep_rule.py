@@ -68,6 +68,10 @@ def test_shapes(shape, maps, programs):
     assert takes_maps(many(leaves(*shape), programs)) == maps
 
 
+def test_few_trips_of_many_programs():
+    assert takes_maps(many(leaves(16, 64, 4, 1), 12000)) and takes_maps(many(leaves(16, 16, 64, 1), 6000))
+
+
 def test_short_work_needs_the_warps():
     """Trips of 8: by maps while every warp has few neighbours, walked where
     24 warps an SM take the batch at once and 16 do not."""
