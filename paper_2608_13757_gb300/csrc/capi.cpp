@@ -364,8 +364,13 @@ static void build_pieces(const sync_batch_desc& d, const LoopInfo* loop, const i
     // program far above the batch's share per warp, speculated otherwise
     const bool bf = !force_spec && (double)pi.n_inst > 4.0 * (2.0 * pi.ne + 1.0) * share;
     bf_init.push_back(bf ? 0 : 1);
-    if (bf) ne_max = std::max(ne_max, pi.ne);
-    else add_cost(h.spec_cost, sum[p], np);
+    if (bf) {
+      ne_max = std::max(ne_max, pi.ne);
+      std::vector<int32_t> body((size_t)(d.prog_loop_ptr[p + 1] - d.prog_loop_ptr[p]));
+      for (int32_t x = 0; x < nx; ++x) h.body_max = std::max(h.body_max, ++body[d.instr_loop[x0 + x]]);
+    } else {
+      add_cost(h.spec_cost, sum[p], np);
+    }
     // the program's instances in the compact scratch of the stored times
     const int64_t first = nx > 0 ? inst_off[x0] : 0;
     for (int32_t j = 0; j < np; ++j) {
@@ -1269,7 +1274,7 @@ static void simulate(const sync_programs* h, sync_thr_mode mode, bool fused, con
     w.pcs.shift = h->piece_shift; w.pcs.vp = h->spec_vp;
     SweepArgs wp = w;
     PieceLaunch L{h->vdep, h->piece_cnt, stored_times(h, true), h->pinst[0], h->n_split, h->n_probed, h->n_spec,
-                  h->spec_cost};
+                  h->spec_cost, h->body_max};
     wp.pcs.probes = h->probes_bf;
     if (h->n_probed > 0) {                         // the probes' histories and stored times
       wp.pcs.phist = probe_history(h, mode);

@@ -517,6 +517,7 @@ struct PieceLaunch {
   int64_t one_len;           // instances of all split programs
   int32_t n_split, n_probed, n_spec;   // split programs; of these barrier-free probed / speculated
   SweepCost spec_cost;       // of the speculated pieces
+  int32_t body_max;          // most records in a loop's body of a probed program
 };
 cudaError_t launch_pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaStream_t s);
 // Barrier scheme by intervals in separate launches, for a batch with split

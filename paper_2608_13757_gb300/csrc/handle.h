@@ -125,6 +125,7 @@ struct sync_programs {
   int64_t pinst[2] = {0, 0};            // instances of the split programs (all, probed)
   mutable int32_t* ptimes[2] = {nullptr, nullptr};   // their stored times, allocated on first use
   int32_t* xeng = nullptr;              // engine per instruction (split batches)
+  int32_t body_max = 0;                 // most records in a loop's body of a probed program
   int32_t nx_max_split = 1;             // most instructions of a split program
   int32_t nsem_max[syncgb::kModes] = {0, 0, 0};
   int32_t ne_max = 1;

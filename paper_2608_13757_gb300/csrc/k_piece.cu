@@ -319,14 +319,20 @@ cudaError_t pieces(const SweepArgs& a, const PieceLaunch& L, int num_sms, cudaSt
     p.ring = sweep_ring(p.sem_cap, p.frame_depth, false);
     if (p.ring < 1) return cudaErrorInvalidConfiguration;
     const size_t smem = sweep_smem_bytes(p.sem_cap, p.frame_depth, p.ring, false);
-    // 128 registers a thread (no spills) and 16 warps per SM, unless 24 warps
-    // take all runs at once and 16 do not: GEMM batches at 80 / 128
-    // registers, 1 program (320 runs) 2.30 / 2.14 ms, 4 3.20 / 3.05, 8 (2560)
-    // 6.1 / 7.4, 12 (3840) 10.9 / 8.5, 20 15.3 / 13.7.
+    // 80 registers a thread and 24 warps per SM, or 128 (no spills) and 16:
+    // a wave of the former takes about as long where the bodies are short,
+    // and longer where their records and spills fill the L1.  80 / 128
+    // registers, ms, bodies of 148 records (GEMM): 4 programs (320 runs each)
+    // 3.23 / 3.10, 8 6.3 / 7.5, 12 12.0 / 8.7, 20 17.6 / 14.1, 40 35.2 / 28.2;
+    // 100 records: 14 10.4 / 8.3, 18 11.0 / 11.7; 16 records: 14 3.3 / 3.2, 18
+    // 4.0 / 4.8, 64 11.6 / 13.7; attention (12) 4 3.5 / 3.1, 24 10.9 / 11.8,
+    // 64 23.6 / 27.4.
     const int64_t runs = (int64_t)p.pcs.n_pieces * p.pcs.probes;
-    const bool one_wave = runs > 2 * kWarps * num_sms && runs <= 3 * kWarps * num_sms;
-    e = one_wave ? launch_items(k_sweep<MODE, false, true, false, true>, p, runs, smem, num_sms, s)
-                 : launch_items(k_sweep<MODE, false, true, false, true, false, false, true>, p, runs, smem, num_sms, s);
+    const auto waves = [&](int64_t ctas) { return (runs + ctas * kWarps * num_sms - 1) / (ctas * kWarps * num_sms); };
+    const double longer = L.body_max <= 64 ? 1.05 : L.body_max <= 128 ? 1.25 : 1.6;
+    e = (double)waves(3) * longer < (double)waves(2)
+            ? launch_items(k_sweep<MODE, false, true, false, true>, p, runs, smem, num_sms, s)
+            : launch_items(k_sweep<MODE, false, true, false, true, false, false, true>, p, runs, smem, num_sms, s);
     if (e != cudaSuccess) return e;
     k_piece_resolve<<<warp_blocks, 256, 0, s>>>(p, L.n_split);
     if ((e = launched()) != cudaSuccess) return e;
