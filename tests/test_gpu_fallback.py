@@ -90,8 +90,8 @@ def test_fallback_random_trees(sg, seed):
 
 
 def test_fallback_beside_sweep_programs(sg):
-    """Fallback programs (per-engine kernel, barrier-free) in one batch with
-    chain programs the sweep runs, and the hand-checked program."""
+    """Fallback programs (their barriers are items of the sweep's plans) in
+    one batch with chain programs, and the hand-checked program."""
     b = workloads.concat([workloads.generate("chain", n_programs=64),
                           workloads.random_trees(31010, 60, workloads.tree_params(**FAR)),
                           nested_program(1), nested_program(2, backward=True)])
@@ -266,4 +266,42 @@ def test_fallback_hand_long_trips(sg):
     for r in (sg.sync_simulate(h, COUNT, thr), sg.sync_simulate_noalloc(h, COUNT, thr),
               sg.sync_simulate_fused(h, COUNT)):
         assert r.status.cpu().tolist()[:1] == [0] and r.makespan.cpu().tolist()[:1] == [10693]
+    h.close()
+
+
+def forward_program(trips, rng):
+    """A loop with a fallback barrier whose first instruction waits for one
+    later in the iteration on another engine: no program order satisfies it,
+    the engines have to be walked each on its own."""
+    b = workloads.ProgramBuilder(3)
+    a = b.loop(0, 0, trips[:1])
+    s = b.loop(a, 0, [trips[1]] * trips[0])
+    n = trips[0] * trips[1]
+    lat = lambda: int(rng.integers(1, 60))
+    c = b.instr(s, 0, 1, lat())
+    x = b.loop(s, 1, rng.integers(0, 4, size=n).tolist())
+    q = b.instr(x, 0, 0, lat())
+    r = b.instr(s, 2, 2, lat())
+    p = b.instr(s, 3, 0, lat())
+    b.dep(p, c, 0)                     # waits forward
+    b.dep(q, r, 1)                     # the fallback barrier
+    b.dep(c, r, 0)
+    return b.batch()
+
+
+def test_fallback_with_waits_forward(sg):
+    """Fallback barriers in the per-engine kernel, to which the sweep leaves
+    programs whose waits point forward in program order; also through the
+    call that allocates nothing."""
+    import torch
+    rng = np.random.default_rng(3)
+    b = with_policy(workloads.concat([forward_program(t, rng) for t in ((1, 1), (2, 3), (3, 20), (1, 70))] +
+                                     [nested_program(1)]), 1)
+    assert (oracle.classify(b).kase == oracle.CASE_BARRIER).sum() == 5
+    h = compare_fallback(sg, b, oracle.sim_params(ii=2, c_branch=3, c_regop=2, c_barrier=17))
+    thr = sg.sync_eval_thresholds(h, PERLOOP)
+    want, got = (f(h, PERLOOP, thr, timeline=True) for f in (sg.sync_simulate, sg.sync_simulate_noalloc))
+    for f in ("status", "makespan", "checksum", "issue", "retire"):
+        assert torch.equal(getattr(got, f), getattr(want, f)), f
+    assert not want.status.cpu().numpy()[:b.n_programs].any()
     h.close()

@@ -661,12 +661,13 @@ def test_alu_reductions_configs(sg, name, n):
 
 
 def test_alu_reductions_in_the_per_engine_kernel(sg):
-    """Programs the sweep hands to the per-engine kernel -- barrier
-    fallbacks (barrier-free), waits on later producers, per-engine trips --
-    with the reductions on."""
+    """Programs the sweep hands to the per-engine kernel -- waits on later
+    producers, with fallback barriers and without, per-engine trips -- with
+    the reductions on, and fallback programs of the sweep."""
     from tests.test_fallback_pins import FAR
-    from tests.test_gpu_fallback import compare_fallback
-    fb = workloads.random_trees(9400, 60, workloads.tree_params(**FAR))
+    from tests.test_gpu_fallback import compare_fallback, forward_program
+    fb = workloads.concat([workloads.random_trees(9400, 60, workloads.tree_params(**FAR)),
+                           forward_program((2, 9), np.random.default_rng(9400))])
     fb.nonalloc_policy = 1
     b = workloads.ProgramBuilder(2)          # a consumer ahead of its producer on another engine
     A = b.loop(0, 0, [3])

@@ -132,10 +132,11 @@ def test_pieces_refuse_waits_into_earlier_pieces(sg, monkeypatch):
 def test_kernel_launch_count(sg, spec, monkeypatch):
     """The library's launch counter: one kernel per threshold and check
     call, two per simulation of unsplit programs (the sweep and the
-    per-engine kernel), and the piece kernels on top where programs are
-    split: barrier scheme validation, runs, composition and fixup;
-    barrier-free validation, then probes (runs, composition) and/or
-    speculation (start, four rounds of runs and acceptance), then fixup."""
+    per-engine kernel), and on top where programs are split the interval
+    kernels in the barrier scheme (classes, schedules, composition, tiles) and
+    the piece kernels barrier-free: validation, then probes (runs,
+    composition) and/or speculation (start, four rounds of runs and
+    acceptance), then fixup."""
     monkeypatch.setenv("SYNCGB_SPLIT_SPEC", spec)
     mode = oracle.PERLOOP
     for name, split in (("depth2", False), ("gemm", True)):

@@ -118,8 +118,7 @@ def test_noalloc_refuses_batches_beyond_its_scratch(sg):
 
 
 def test_noalloc_with_the_barrier_fallback(sg):
-    """Programs with fallback barriers (handed to the per-engine kernel,
-    barrier-free) beside ordinary ones: the same results as sync_simulate,
+    """Programs with fallback barriers beside ordinary ones: the same results as sync_simulate,
     and the unrolled variant refused here too."""
     import torch
     from tests.test_fallback_pins import FAR, nested_program
