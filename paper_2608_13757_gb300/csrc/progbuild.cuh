@@ -1058,11 +1058,12 @@ struct ProgBuilder {
           add_item(make_int4(ITEM_LOOP, l0 + m, FILL ? O.lflag[l0 + m] : 0, 0));
         }
       }
-      // a fallback barrier ends the iteration: not a leaf for the sweep's loops
+      // a fallback barrier ends the iteration (such a loop has a child loop, the
+      // producer's: it is no leaf)
       if (S.fbar[l0 + l]) add_item(make_int4(ITEM_BARRIER, 0, 0, 0));
       // a short body with no child loop: a template of several iterations
       const int32_t L = bp[l + 1] - bp[l];
-      if (nloops == 0 && nseg == 1 && L >= 1 && L <= 16 && !S.fbar[l0 + l]) {
+      if (nloops == 0 && nseg == 1 && L >= 1 && L <= 16) {
         const int32_t k = 32 / L;
         if constexpr (!FILL) {                    // COUNT: every record in each of k copies
           c[BC_LANES] += (int64_t)k * L;
@@ -1139,8 +1140,6 @@ struct ProgBuilder {
         if (e - b == 1 && O.plan[b].x == ITEM_SEG) {
           if (O.plan[b].z == 1) bf = bb = O.plan[b].y;
           if (O.plan[b].w >= 0) bf = O.plan[b].w;
-        } else if (e - b == 2 && O.plan[b].x == ITEM_SEG && O.plan[b].z == 1 && O.plan[b + 1].x == ITEM_BARRIER) {
-          bb = O.plan[b].y;                       // the barrier scheme has that barrier already
         }
         const int64_t rp = S.srp[sr(m, 0)];
         O.paux[i] = make_int4((int32_t)(uint32_t)(rp & 0xffffffffu), (int32_t)(rp >> 32), bf, bb);
