@@ -21,12 +21,17 @@
 //            with its class, every instance's times and checksum term;
 //   a program with a wait outside its class, or whose segment cannot be
 //   scheduled, is swept instead (k_sweep), which gives its verdict.
-// Nothing is serial but a program's plan.  What bounds a tile is its integer
-// instructions -- 14 per instance and lane for the times and the checksum, 7
-// per wait -- and the latency of its prologue.  Barrier simulation, walked /
-// by intervals: 65536 chain programs (1.25e9 instances) 15.1 / 4.7 ms (plans
-// 0.6, waits 1.6, times 2.2), 65536 sync-bound ones 35.2 / 3.6, 256 attention
-// programs 14.3 / 0.84, 4096 depth-2 ones 4.1 / 0.34, the GEMM 2.7 / 0.16.
+// A program whose walk takes less than its plan is walked too (enc.h has the
+// rule).  Nothing is serial but a program's plan.  What bounds a tile is its
+// integer instructions -- 14 per instance and lane for the times and the
+// checksum, 7 per wait -- and the latency of its prologue.  Barrier simulation,
+// walked / by intervals: 65536 chain programs (1.25e9 instances) 15.1 / 4.7 ms
+// (plans 0.6, waits 1.6, times 2.2), 65536 sync-bound ones 35.2 / 3.6, 256
+// attention programs 14.3 / 0.87, 4096 depth-2 ones 4.1 / 0.36, the GEMM 2.7 /
+// 0.17.  These are repeated calls: the first one on a handle also lays out the
+// positions in the engines' streams, which depend on the batch alone (chain
+// 5.1 ms, pool allocation included; 6001 branching trees 0.7 instead of 0.5).
+// On every call they would take 0.34 ms of the chain's, 0.17 of the trees'.
 #pragma once
 
 #include "cost.cuh"
@@ -278,7 +283,7 @@ __device__ __forceinline__ void bar_pub(const SweepArgs& a, const DepInfo& D, co
   }
 }
 
-// The counts of program p's starts and sums, once per handle.
+// The counts of program p's starts and sums (q >= 1), once per handle.
 __device__ __forceinline__ void bar_counts(const SweepArgs& a, int p, const ProgInfo& pi, int lane) {
   if (a.bar.counted[p]) return;
   bar_fill(a, pi, 1, 1 + pi.ne, lane);

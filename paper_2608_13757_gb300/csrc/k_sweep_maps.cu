@@ -1,5 +1,5 @@
-// Schedule simulator, program-order sweep, barrier-free by chunk maps
-// (sweep.cuh): the launcher for batches whose time is their longest programs'.
+// Schedule simulator, program-order sweep, barrier-free, trips by their maps
+// (trip.cuh): the launcher for the batches that sweep_maps() sends here.
 #include "sweep.cuh"
 
 namespace syncgb {

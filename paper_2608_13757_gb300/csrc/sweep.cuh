@@ -24,8 +24,8 @@
 //   - a threshold beyond every increment up to this chunk points forward in
 //     program order: the program is handed to the per-engine kernel.
 // Trips of loops around straight lines go by their max-plus maps where that
-// pays (trip.cuh, sweep_maps in enc.h); the barrier scheme by intervals
-// (bar.cuh), its walk only for what those leave.
+// pays (trip.cuh, sweep_maps in k_sweep.cu); the barrier scheme by intervals
+// (bar.cuh), its walk for what those leave and where it takes less.
 // A loop whose body is one chunk runs all its iterations in a tight loop
 // with the lanes' records in registers and the next iteration's thresholds
 // in flight.  Barriers (barrier scheme) are a warp maximum of the engines'
@@ -884,8 +884,8 @@ __device__ __forceinline__ int run_loop(const SweepArgs& a, const WarpSmem& S, c
 // PieceArgs) instead of whole programs: item = piece * probes + probe; the
 // walk starts inside the body of the piece's loop L at its first iteration
 // start and ends after its last iteration.
-// BAR (barrier scheme): programs by intervals (bar.cuh), and by the walk only
-// those the intervals leave.  MAPS (barrier-free): trips by their maps
+// BAR (barrier scheme): programs by intervals (bar.cuh), and by the walk those
+// the intervals leave or whose walk takes less.  MAPS (barrier-free): trips by their maps
 // (trip.cuh).  REGS: 128 registers and 16 warps per SM without maps.
 template <int MODE, bool BB, bool TL, bool FUSED, bool PIECE = false, bool BAR = false, bool MAPS = false, bool REGS = false>
 __global__ void __launch_bounds__(kWarps * 32, MAPS || REGS ? 2 : BAR ? kBarCtas : 3) k_sweep(const __grid_constant__ SweepArgs a) {

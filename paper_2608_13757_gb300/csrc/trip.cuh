@@ -24,8 +24,8 @@
 // bounds it is one warp's dependent instructions: an iteration of 17 records
 // took 1500 cycles walked; with 11 inputs phase 1 takes 119, phase 2 184 per
 // record and 32 iterations, the comparison 565 to 1100 a batch.  Barrier-free,
-// walked / by maps: 4096 depth-2 programs 4.8 / 1.1 ms, 777 chain programs
-// 9.3 / 5.9, 256 attention programs (pieces) 14.9 / 7.9, 65536 sync-bound
+// walked / by maps: 4096 depth-2 programs 4.9 / 1.1 ms, 777 chain programs
+// 9.2 / 6.2, 256 attention programs (pieces) 14.9 / 7.9, 65536 sync-bound
 // ones 34.0 / 12.5.  Two records per half warp for short trips, skipping a
 // record's groups without weights, and unrolling by 4 were no faster.
 #pragma once
