@@ -28,10 +28,10 @@
 // walked / by intervals: 65536 chain programs (1.25e9 instances) 15.1 / 4.7 ms
 // (plans 0.6, waits 1.6, times 2.2), 65536 sync-bound ones 35.2 / 3.6, 256
 // attention programs 14.3 / 0.87, 4096 depth-2 ones 4.1 / 0.36, the GEMM 2.7 /
-// 0.17.  These are repeated calls: the first one on a handle also lays out the
+// 0.18.  These are repeated calls: the first one on a handle also lays out the
 // positions in the engines' streams, which depend on the batch alone (chain
-// 5.1 ms, pool allocation included; 6001 branching trees 0.7 instead of 0.5).
-// On every call they would take 0.34 ms of the chain's, 0.17 of the trees'.
+// 5.1 ms, pool allocation included; 3000 branching trees 0.62 instead of 0.35,
+// cold caches included).  On every call they would take 0.34 ms of the chain's.
 #pragma once
 
 #include "cost.cuh"

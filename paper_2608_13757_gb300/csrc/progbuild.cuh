@@ -211,6 +211,24 @@ PB_HD void pb_sort(int64_t* a, int64_t n) {
   }
 }
 
+// A walked leaf iteration's share of its chunk (sweep_cost): 1300 cycles a
+// chunk without waits inside it, else 2300 with 2 or 3 iterations, 2000 with 4
+// or 5, 1500 with more and with one.
+struct LeafCosts {
+  int32_t of[2][33];
+  constexpr const int32_t* operator[](int inner) const { return of[inner]; }
+};
+constexpr LeafCosts leaf_costs() {
+  LeafCosts c{};
+  for (int len = 1; len <= 32; ++len) {
+    const int copies = len <= 16 ? 32 / len : 1;
+    c.of[0][len] = 1300 / copies;
+    c.of[1][len] = (len > 16 ? 1500 : len > 8 ? 2300 : len > 5 ? 2000 : 1500) / copies;
+  }
+  return c;
+}
+constexpr LeafCosts kLeafCost = leaf_costs();
+
 template <bool FILL>
 struct ProgBuilder {
   const BuildArgs& A;
@@ -1161,9 +1179,8 @@ struct ProgBuilder {
   // few neighbours: walked, and with trips by their maps where the sweep can
   // build and use one (SweepCost in enc.h; trip.cuh has the conditions).
   // Measured on one loop of 4 to 40 records, trips of 8 to 64: a loop
-  // statement 1400; a chunk of records 2300 with 2 or 3 iterations in it, 2000
-  // with 4 or 5, 1500 with more and with one, each 1300 without waits inside
-  // it, 2600 outside a leaf loop; a batch of up to 32 iterations by a map 1900
+  // statement 1400; a chunk of a leaf loop 1300 to 2300 (kLeafCost) and half a
+  // chunk of several iterations a visit, 2600 elsewhere; a batch of up to 32 iterations by a map 1900
   // + 246 a record, and 34 + 5.2 a record for each iteration; building the
   // map 2000 an input.  (0.1 us a program, 1% of a chain batch's load.)
   PB_HD void sweep_cost() {
@@ -1203,8 +1220,7 @@ struct ProgBuilder {
       const bool inner = w >> 16 > (w & (kMany - 1)) || (len <= 10 && (w & kNear));
       if (nloops > 0) c += len > 0 ? t * (cuts + chunks) * 2600 : 0;
       else if (len > 32) c += t * chunks * 2600;
-      else if (len > 16) c += t * (inner ? 1500 : 1300);
-      else if (len > 0) c += t * ((!inner ? 1300 : len > 8 ? 2300 : len > 5 ? 2000 : 1500) / (32 / len)) + np * 1000;
+      else c += t * kLeafCost[inner][len] + (len > 0 && len <= 16 ? np * 1000 : 0);
       cost[(int64_t)l * ne] = c;
       cand[l] = S.fbar[l0 + l] ? kOut : 0;
     }
@@ -1244,13 +1260,12 @@ struct ProgBuilder {
       // loop takes its place, and begins with kTripLearn walked iterations
       int32_t a = l;
       while (a != 0 && (cand[par[a]] & ~kOut) == 1) a = par[a];
-      const double visits = (double)n_parent(l, 0), runs = a == 0 ? 1 : (double)tot(par[a], 0);
-      const double trip = (double)tot(l, 0) / visits;
-      const double walked = (double)(int64_t)(trip >= kTripLearn ? 1 : (kTripLearn + trip - 1) / trip) * runs;
-      if (walked >= visits) continue;
-      const double batches = (double)(((int64_t)trip + 31) / 32);
-      const double one = batches * (1900 + 246 * n_rec) + trip * (34 + 5.2 * n_rec);
-      map += runs * 2000 * inputs + (visits - walked) * (one - ((double)c / visits - 1400));
+      const int64_t v = n_parent(l, 0), t = tot(l, 0), runs = a == 0 ? 1 : tot(par[a], 0);
+      const int64_t walked = t >= kTripLearn * v ? runs : runs * ((kTripLearn * v + t - 1) / t);   // visits
+      if (walked >= v) continue;
+      const int64_t batches = t <= 32 * v ? v : (t + 31 * v) / (32 * v) * v;
+      const double mapped = (double)(batches * (1900 + 246 * n_rec)) + (double)t * (34 + 5.2 * n_rec);
+      map += (double)(runs * 2000 * inputs) + (mapped - (double)(c - 1400 * v)) * ((double)(v - walked) / (double)v);
     }
     sm.map = (int64_t)map;
   }
